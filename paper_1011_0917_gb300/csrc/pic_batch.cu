@@ -54,7 +54,7 @@ __device__ __forceinline__ void batch_tiles(const PushArgs<real> *__restrict__ r
 }
 
 template <typename real, int DIM, int S, int TX, int TY, int TZ, bool REL>
-__global__ void __launch_bounds__(kBlock, MinBlocks<real>::value)
+__global__ void __launch_bounds__((BlockOf<real, DIM>::value), (MinBlocks<real, DIM>::value))
     push_batch_kernel(const PushArgs<real> *__restrict__ runs, const int64_t *__restrict__ start, int n,
                       unsigned *queue)
 {
@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<real>::value)
 }
 
 template <typename real, int DIM, int S, int TX, int TY, int TZ, bool REL>
-__global__ void __launch_bounds__(kBlock)
+__global__ void __launch_bounds__((BlockOf<real, DIM>::value))
     ion_batch_kernel(const PushArgs<real> *__restrict__ runs, const int64_t *__restrict__ start, int n,
                      unsigned *queue)
 {
@@ -80,12 +80,12 @@ void launch_push_batch(const void *args, const int64_t *start, int n, int64_t to
     auto k = IONS ? ion_batch_kernel<real, DIM, S, TX, TY, TZ, REL> : push_batch_kernel<real, DIM, S, TX, TY, TZ, REL>;
     if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int per_sm = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kBlock, smem) != cudaSuccess || per_sm < 1)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, BlockOf<real, DIM>::value, smem) != cudaSuccess || per_sm < 1)
         per_sm = 1;
     int64_t grid = (int64_t)per_sm * device_sms();
     if (grid > total) grid = total;
     if (grid < 1) grid = 1;
-    k<<<(unsigned)grid, kBlock, smem, s>>>(static_cast<const PushArgs<real> *>(args), start, n, queue);
+    k<<<(unsigned)grid, BlockOf<real, DIM>::value, smem, s>>>(static_cast<const PushArgs<real> *>(args), start, n, queue);
 }
 
 // every kernel configuration the single-run launchers dispatch to

@@ -52,8 +52,10 @@ int ceil_log2(int64_t n)
     return b;
 }
 
-struct SideLayout {       // byte offsets of the attribute arrays within one side
-    size_t off[kAttrs];   // ox oy oz w ux uy uz cell id dz (SIZE_MAX: absent)
+struct SideLayout {       // one side of a species (attributes ox oy oz w ux uy uz cell id dl*)
+    size_t off[kAttrs];   // as flat arrays (staging of uploads and downloads): byte offset (SIZE_MAX: absent)
+    size_t boff[kAttrs];  // as blocks of 32 records: byte offset of the attribute's row in a block (id: its array)
+    size_t rb;            // bytes of a block
     size_t bytes;
 };
 
@@ -204,14 +206,25 @@ static void *eb_other(pic_ctx *c, int comp)
     return c->fields + (size_t)comp * c->g.ncomp * c->es;
 }
 
+// the attribute pointers of a side: its blocks, or (flat) its arrays as a
+// staging area
+static void side_raw(pic_ctx *c, int sp, int sidx, bool flat, void *out[kAttrs])
+{
+    const SideLayout &L = c->side[sp];
+    unsigned char *base = c->species[sp] + (size_t)sidx * L.bytes;
+    for (int a = 0; a < kAttrs; ++a)
+        out[a] = L.off[a] == SIZE_MAX ? nullptr : (void *)(base + (flat ? L.off[a] : L.boff[a]));
+}
+
 template <typename real>
-static Species<real> species_view(pic_ctx *c, int sp, int sidx)
+static Species<real> species_view(pic_ctx *c, int sp, int sidx, bool flat = false)
 {
     Species<real> s{};
-    unsigned char *base = c->species[sp] + (size_t)sidx * c->side[sp].bytes;
-    auto at = [&](int a) -> void * {
-        return c->side[sp].off[a] == SIZE_MAX ? nullptr : (void *)(base + c->side[sp].off[a]);
-    };
+    void *p[kAttrs];
+    side_raw(c, sp, sidx, flat, p);
+    auto at = [&](int a) -> void * { return p[a]; };
+    s.sr = flat ? 32 : (int)(c->side[sp].rb / sizeof(real));
+    s.sc = flat ? 32 : (int)(c->side[sp].rb / 4);
     s.ox = (real *)at(0);
     s.oy = (real *)at(1);
     s.oz = (real *)at(2);
@@ -225,13 +238,6 @@ static Species<real> species_view(pic_ctx *c, int sp, int sidx)
     s.dly = (real *)at(10);
     s.dlz = (real *)at(11);
     return s;
-}
-
-static void side_raw(pic_ctx *c, int sp, int sidx, void *out[kAttrs])
-{
-    unsigned char *base = c->species[sp] + (size_t)sidx * c->side[sp].bytes;
-    for (int a = 0; a < kAttrs; ++a)
-        out[a] = c->side[sp].off[a] == SIZE_MAX ? nullptr : (void *)(base + c->side[sp].off[a]);
 }
 
 static cudaMemcpyKind kind_out(int dst_is_device) { return dst_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost; }
@@ -391,6 +397,16 @@ extern "C" pic_status pic_init_grid(const pic_grid_params *p, pic_ctx **out)
             o += align_up((size_t)c->slots * attr_size(c, a));
         }
         L.bytes = o;
+        // blocks of 32 records in the order of Rec (the cell words last, ids
+        // in an array behind the blocks); they take no more than the arrays
+        size_t q = 0;
+        for (int a : {0, 1, 2, 3, 4, 5, 6, 9, 10, 11, 7})
+            if (L.off[a] != SIZE_MAX) {
+                L.boff[a] = q;
+                q += 32 * attr_size(c, a);
+            }
+        L.rb = q;
+        L.boff[8] = (size_t)(c->slots / 32) * q;
         c->species_bytes[sp] = (sp == 1 && !c->ions_species) ? 0 : 2 * o;
     }
     size_t o = 0;
@@ -496,10 +512,14 @@ static void fill_inject_common(pic_ctx *c, InjectArgs &a)
     a.drift_ions = (p.ions && c->ions_species) ? 1 : 0;
     a.paired = (a.drift_ions && !c->p.explicit_ions) ? 1 : 0;
     a.precision = c->p.precision;
-    side_raw(c, 0, c->cur[0], a.sp_e);
+    side_raw(c, 0, c->cur[0], false, a.sp_e);
+    a.sr_e = (int)(c->side[0].rb / (size_t)c->es);
+    a.sc_e = (int)(c->side[0].rb / 4);
+    a.sr_i = (int)(c->side[1].rb / (size_t)c->es);
+    a.sc_i = (int)(c->side[1].rb / 4);
     a.hi_e = counts(c, 0, c->cur[0], 1);
     if (a.drift_ions) {
-        side_raw(c, 1, c->cur[1], a.sp_i);
+        side_raw(c, 1, c->cur[1], false, a.sp_i);
         a.hi_i = counts(c, 1, c->cur[1], 1);
     } else {
         for (int q = 0; q < kAttrs; ++q) a.sp_i[q] = nullptr;
@@ -588,7 +608,7 @@ static pic_status bucket_staged(pic_ctx *c, int sp, int64_t n)
     const int stage = c->cur[sp] ^ 1;
     BucketArgs<real> b{};
     b.g = c->g;
-    b.src = species_view<real>(c, sp, stage);
+    b.src = species_view<real>(c, sp, stage, true);
     b.dst = species_view<real>(c, sp, c->cur[sp]);
     b.n = n;
     b.dst_hi = counts(c, sp, c->cur[sp], 1);
@@ -603,7 +623,7 @@ template <typename real>
 static pic_status upload_flat(pic_ctx *c, int sp, int64_t n, const void *const cols[kAttrs], int src_is_device)
 {
     void *dst[kAttrs];
-    side_raw(c, sp, c->cur[sp] ^ 1, dst);
+    side_raw(c, sp, c->cur[sp] ^ 1, true, dst);
     for (int a = 0; a < kAttrs; ++a) {
         if (!dst[a]) continue;
         const size_t bytes = (size_t)n * attr_size(c, a);
@@ -1778,7 +1798,7 @@ static pic_status compact_t(pic_ctx *c, int sp, int64_t &n)
     CompactArgs<real> a{};
     a.g = c->g;
     a.src = species_view<real>(c, sp, c->cur[sp]);
-    a.dst = species_view<real>(c, sp, c->cur[sp] ^ 1);
+    a.dst = species_view<real>(c, sp, c->cur[sp] ^ 1, true);
     a.lo = counts(c, sp, c->cur[sp], 0);
     a.hi = counts(c, sp, c->cur[sp], 1);
     a.offset = d_off;
@@ -1795,7 +1815,7 @@ static pic_status download_species(pic_ctx *c, int sp, int64_t &n, std::vector<s
     pic_status s = compact_t<real>(c, sp, n);
     if (s != PIC_OK) return s;
     void *col[kAttrs];
-    side_raw(c, sp, c->cur[sp] ^ 1, col);
+    side_raw(c, sp, c->cur[sp] ^ 1, true, col);
     h.assign(kAttrs, {});
     for (int a = 0; a < kAttrs; ++a) {
         if (!col[a]) continue;
@@ -2043,7 +2063,7 @@ static pic_status get_state_t(pic_ctx *c, unsigned char *dst, size_t dst_bytes, 
     }
     for (int sp = 0; sp < (c->ions_species ? 2 : 1); ++sp) {
         void *col[kAttrs];
-        side_raw(c, sp, c->cur[sp] ^ 1, col);
+        side_raw(c, sp, c->cur[sp] ^ 1, true, col);
         for (int a = 0; a < kAttrs; ++a) {
             if (!col[a]) continue;
             const size_t b = (size_t)n[sp] * attr_size(c, a);

@@ -75,9 +75,10 @@ __device__ __forceinline__ void to_cell(double x, double h, int n, bool periodic
 }
 
 template <typename real>
-__device__ __forceinline__ void store(void *const sp[kAttrs], int64_t d, real ox, real oy, real oz, real w, int32_t cell,
+__device__ __forceinline__ void store(void *const sp[kAttrs], int sr, int sc, int64_t d0, real ox, real oy, real oz, real w, int32_t cell,
                                       int64_t id, bool electron, bool dim3)
 {
+    const int64_t d = (d0 >> 5) * sr + (d0 & 31);
     static_cast<real *>(sp[0])[d] = ox;
     if (dim3) static_cast<real *>(sp[1])[d] = oy;
     static_cast<real *>(sp[2])[d] = oz;
@@ -87,8 +88,8 @@ __device__ __forceinline__ void store(void *const sp[kAttrs], int64_t d, real ox
         static_cast<real *>(sp[5])[d] = real(0);
         static_cast<real *>(sp[6])[d] = real(0);
     }
-    static_cast<int32_t *>(sp[7])[d] = cell;
-    if (sp[8]) static_cast<int64_t *>(sp[8])[d] = id;
+    static_cast<int32_t *>(sp[7])[(d0 >> 5) * sc + (d0 & 31)] = cell;
+    if (sp[8]) static_cast<int64_t *>(sp[8])[d0] = id;
     if (electron) {  // relative form: on its reference
         for (int q = 9; q < kAttrs; ++q)
             if (sp[q]) static_cast<real *>(sp[q])[d] = real(0);
@@ -196,11 +197,11 @@ __device__ __forceinline__ void inject_body(const InjectArgs &a, const int64_t b
         const int32_t cell = pack_cell(a.g, ci, cj, ck);
         const int32_t ecell = (int32_t)((uint32_t)cell | (a.paired ? kPaired : 0u));
         if (re < a.g.cap)
-            store<real>(a.sp_e, dest * (int64_t)a.g.cap + (a.g.cap - 1 - re), ox, oy, oz, wr, ecell, L, true, dim3);
+            store<real>(a.sp_e, a.sr_e, a.sc_e, dest * (int64_t)a.g.cap + (a.g.cap - 1 - re), ox, oy, oz, wr, ecell, L, true, dim3);
         else atomicOr(a.err, ERR_CAPACITY);
         if (a.drift_ions && !a.paired) {
             if (ri < a.g.cap)
-                store<real>(a.sp_i, dest * (int64_t)a.g.cap + (a.g.cap - 1 - ri), ox, oy, oz, wr, cell, L, false,
+                store<real>(a.sp_i, a.sr_i, a.sc_i, dest * (int64_t)a.g.cap + (a.g.cap - 1 - ri), ox, oy, oz, wr, cell, L, false,
                             dim3);
             else atomicOr(a.err, ERR_CAPACITY);
         }

@@ -6,8 +6,11 @@
 //            array index (i, j, k): Ex (i+1/2, j, k), Ey (i, j+1/2, k),
 //            Ez (i, j, k+1/2), Bx (i, j+1/2, k+1/2), By (i+1/2, j, k+1/2),
 //            Bz (i+1/2, j+1/2, k); J like E.
-//   species: per species two "sides" (double buffer).  A side is a structure
-//            of arrays with `slots` entries per attribute; tile t owns slots
+//   species: per species two "sides" (double buffer).  A side holds `slots`
+//            records in blocks of 32: a block is 32 values of the first
+//            attribute, 32 of the next, ... (Rec), so that the 32 records a
+//            warp works on are one contiguous piece (1 KB for an FP32
+//            electron in 3D) reached with one address.  Tile t owns slots
 //            [t*cap, (t+1)*cap) and keeps its particles in two runs: a bottom
 //            run [0, lo) that the tile's own CTA writes (particles that stayed
 //            in the tile, counted in shared memory) and a top run
@@ -56,6 +59,11 @@ struct Geom {
 // id dlx dly dlz (absent ones are null)
 constexpr int kAttrs = 12;
 
+// Record d of an attribute is at pointer[r(d)] (the cell word at cell[c(d)]):
+// in a side of the store the pointers are the attribute's row of block 0 and
+// sr, sc the elements from one block to the next; in a flat list (staging of
+// uploads and downloads, one array per attribute) sr = sc = 32, so r(d) =
+// c(d) = d.  Ids are a plain array in both.
 template <typename real>
 struct Species {
     real *ox, *oy, *oz, *w;     // oy is null in 2D
@@ -63,6 +71,22 @@ struct Species {
     int32_t *cell;
     int64_t *id;                // null unless ids are tracked
     real *dlx, *dly, *dlz;      // relative positions only (see rel_actual); dly null in 2D
+    int sr, sc;
+    __host__ __device__ __forceinline__ int64_t r(int64_t d) const { return (d >> 5) * sr + (d & 31); }
+    __host__ __device__ __forceinline__ int64_t c(int64_t d) const { return (d >> 5) * sc + (d & 31); }
+};
+
+// Byte offsets of the attribute rows in a block of 32 records and the block's
+// size RB: reals ox oy oz w, for electrons ux uy uz, in relative form dlx dly
+// dlz (oy, dly in 3D only), then the cell words.
+template <typename real, int DIM, bool ELECTRON, bool REL>
+struct Rec {
+    static constexpr int NR = DIM + 1 + (ELECTRON ? 3 : 0) + (ELECTRON && REL ? DIM : 0);
+    static constexpr int ROW = 32 * (int)sizeof(real);
+    static constexpr int OX = 0, OY = ROW, OZ = (DIM - 1) * ROW, W = DIM * ROW;
+    static constexpr int UX = (DIM + 1) * ROW, UY = UX + ROW, UZ = UX + 2 * ROW;
+    static constexpr int DLX = (DIM + 4) * ROW, DLY = DLX + ROW, DLZ = DLX + (DIM - 1) * ROW;
+    static constexpr int CELL = NR * ROW, RB = CELL + 128;
 };
 
 // Relative positions of an electron record.  In a strongly boosted frame the
@@ -485,6 +509,7 @@ struct InjectArgs {      // lattice load / boosted injection, FP64
     int precision;      // 0 float, 1 double
     void *sp_e[kAttrs];  // ox oy oz w ux uy uz cell id dlx dly dlz of the electron side
     void *sp_i[kAttrs];  // same for the ion side (ux..uz, dl* unused)
+    int sr_e, sc_e, sr_i, sc_i;  // elements from one block of 32 records to the next (reals, cell words)
     int *hi_e, *hi_i;    // top-run lengths of the electron / ion sides
     unsigned *err;
     // fixed-order ("flat") output of an adjoint run (flat_base >= 0, 2D):

@@ -7,7 +7,7 @@
 namespace pic {
 
 template <typename real, int DIM, int S, int TX, int TY, int TZ, bool REL>
-__global__ void __launch_bounds__(kBlock, MinBlocks<real>::value) push_kernel(PushArgs<real> a)
+__global__ void __launch_bounds__((BlockOf<real, DIM>::value), (MinBlocks<real, DIM>::value)) push_kernel(PushArgs<real> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     for (int64_t t = blockIdx.x; t < a.g.ntiles; t += gridDim.x) push_tile<real, DIM, S, TX, TY, TZ, REL>(a, t, smem_raw);
@@ -16,7 +16,7 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<real>::value) push_kernel(Pu
 // ----------------------------------------------------- drifting-ion kernel
 
 template <typename real, int DIM, int S, int TX, int TY, int TZ, bool REL>
-__global__ void __launch_bounds__(kBlock) ion_kernel(PushArgs<real> a)
+__global__ void __launch_bounds__((BlockOf<real, DIM>::value)) ion_kernel(PushArgs<real> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     for (int64_t t = blockIdx.x; t < a.g.ntiles; t += gridDim.x) ion_tile<real, DIM, S, TX, TY, TZ, REL>(a, t, smem_raw);
@@ -32,7 +32,7 @@ static void launch_push_z(const PushArgs<real> &a, bool ions, cudaStream_t s)
     auto k = ions ? ion_kernel<real, DIM, S, TX, TY, TZ, REL> : push_kernel<real, DIM, S, TX, TY, TZ, REL>;
     if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const int64_t grid = a.g.ntiles < 2147483647LL ? a.g.ntiles : 2147483647LL;
-    k<<<(unsigned)grid, kBlock, smem, s>>>(a);
+    k<<<(unsigned)grid, BlockOf<real, DIM>::value, smem, s>>>(a);
 }
 
 // records in relative form (and their ions) take the REL kernels
@@ -85,8 +85,9 @@ __global__ void window_particles_kernel(Geom g, Species<real> in, Species<real> 
     const int n = n_lo + n_hi;
     const uint32_t dk = (uint32_t)S << (g.bx + g.by);
     for (int p = threadIdx.x; p < n; p += blockDim.x) {
-        const int64_t d = bucket_slot(t, g.cap, n_lo, n_hi, p);
-        const int64_t s = d + m * ntxy * (int64_t)g.cap;
+        const int64_t d0 = bucket_slot(t, g.cap, n_lo, n_hi, p);
+        const int64_t s0 = d0 + m * ntxy * (int64_t)g.cap;
+        const int64_t d = out.r(d0), s = in.r(s0);
         out.ox[d] = in.ox[s];
         if (g.dim == 3) out.oy[d] = in.oy[s];
         out.oz[d] = in.oz[s];
@@ -101,8 +102,8 @@ __global__ void window_particles_kernel(Geom g, Species<real> in, Species<real> 
             if (in.dly) out.dly[d] = in.dly[s];
             out.dlz[d] = in.dlz[s];
         }
-        out.cell[d] = (int32_t)((uint32_t)in.cell[s] - dk);  // keeps the pair bit
-        if (in.id) out.id[d] = in.id[s];
+        out.cell[out.c(d0)] = (int32_t)((uint32_t)in.cell[in.c(s0)] - dk);  // keeps the pair bit
+        if (in.id) out.id[d0] = in.id[s0];
     }
 }
 
@@ -133,7 +134,7 @@ __global__ void bucket_kernel(BucketArgs<real> a)
             atomicOr(a.err, ERR_CAPACITY);
             continue;
         }
-        const int64_t d = dest * (int64_t)a.g.cap + (a.g.cap - 1 - r);
+        const int64_t d0 = dest * (int64_t)a.g.cap + (a.g.cap - 1 - r), d = a.dst.r(d0);
         a.dst.ox[d] = a.src.ox[p];
         if (a.dst.oy) a.dst.oy[d] = a.src.oy[p];
         a.dst.oz[d] = a.src.oz[p];
@@ -148,8 +149,8 @@ __global__ void bucket_kernel(BucketArgs<real> a)
             if (a.dst.dly) a.dst.dly[d] = a.src.dly[p];
             a.dst.dlz[d] = a.src.dlz[p];
         }
-        a.dst.cell[d] = a.src.cell[p];
-        if (a.dst.id) a.dst.id[d] = a.src.id ? a.src.id[p] : 0;
+        a.dst.cell[a.dst.c(d0)] = a.src.cell[p];
+        if (a.dst.id) a.dst.id[d0] = a.src.id ? a.src.id[p] : 0;
     }
 }
 
@@ -171,7 +172,7 @@ __global__ void compact_kernel(CompactArgs<real> a)
         const int n = n_lo + n_hi;
         const int64_t o = a.offset[t];
         for (int p = threadIdx.x; p < n; p += blockDim.x) {
-            const int64_t s = bucket_slot(t, a.g.cap, n_lo, n_hi, p), d = o + p;
+            const int64_t s0 = bucket_slot(t, a.g.cap, n_lo, n_hi, p), s = a.src.r(s0), d = o + p;
             a.dst.ox[d] = a.src.ox[s];
             if (a.src.oy) a.dst.oy[d] = a.src.oy[s];
             a.dst.oz[d] = a.src.oz[s];
@@ -186,8 +187,8 @@ __global__ void compact_kernel(CompactArgs<real> a)
                 if (a.src.dly) a.dst.dly[d] = a.src.dly[s];
                 a.dst.dlz[d] = a.src.dlz[s];
             }
-            a.dst.cell[d] = a.src.cell[s];
-            if (a.src.id) a.dst.id[d] = a.src.id[s];
+            a.dst.cell[d] = a.src.cell[a.src.c(s0)];
+            if (a.src.id) a.dst.id[d] = a.src.id[s0];
         }
     }
 }
@@ -235,7 +236,7 @@ __global__ void __launch_bounds__(256) sort_cells_kernel(SortArgs<real> a)
         if (sorted) {
             for (int p = tid; p < n; p += blockDim.x) {
                 int ci, cj, ck;
-                unpack_cell(g, a.in.cell[bucket_slot(t, g.cap, n_lo, n_hi, p)], ci, cj, ck);
+                unpack_cell(g, a.in.cell[a.in.c(bucket_slot(t, g.cap, n_lo, n_hi, p))], ci, cj, ck);
                 int li = ci - lox, lj = cj - loy, lk = ck - loz;
                 if (li < 0 || li >= (1 << g.lt[0]) || lj < 0 || lj >= (1 << g.lt[1]) || lk < 0 ||
                     lk >= (1 << g.lt[2])) {
@@ -268,8 +269,8 @@ __global__ void __launch_bounds__(256) sort_cells_kernel(SortArgs<real> a)
             __syncthreads();
         }
         for (int p = tid; p < n; p += blockDim.x) {
-            const int64_t s = bucket_slot(t, g.cap, n_lo, n_hi, p);
-            const int64_t d = t * (int64_t)g.cap + (sorted ? atomicAdd(&cnt[key[p]], 1) : p);
+            const int64_t s0 = bucket_slot(t, g.cap, n_lo, n_hi, p), s = a.in.r(s0);
+            const int64_t d0 = t * (int64_t)g.cap + (sorted ? atomicAdd(&cnt[key[p]], 1) : p), d = a.out.r(d0);
             a.out.ox[d] = a.in.ox[s];
             if (a.in.oy) a.out.oy[d] = a.in.oy[s];
             a.out.oz[d] = a.in.oz[s];
@@ -284,8 +285,8 @@ __global__ void __launch_bounds__(256) sort_cells_kernel(SortArgs<real> a)
                 if (a.in.dly) a.out.dly[d] = a.in.dly[s];
                 a.out.dlz[d] = a.in.dlz[s];
             }
-            a.out.cell[d] = a.in.cell[s];
-            if (a.in.id) a.out.id[d] = a.in.id[s];
+            a.out.cell[a.out.c(d0)] = a.in.cell[a.in.c(s0)];
+            if (a.in.id) a.out.id[d0] = a.in.id[s0];
         }
         if (tid == 0) {
             a.out_lo[t] = n;
@@ -312,10 +313,11 @@ __global__ void rho_kernel(Geom g, Species<real> sp, const int *lo, const int *h
         bucket_counts(lo, hi, t, g.cap, n_lo, n_hi, nullptr);
         const int n = n_lo + n_hi;
         for (int p = threadIdx.x; p < n; p += blockDim.x) {
-            const int64_t s = bucket_slot(t, g.cap, n_lo, n_hi, p);
-            if ((uint32_t)sp.cell[s] & kPaired) continue;  // with its ion: no net charge
+            const int64_t s0 = bucket_slot(t, g.cap, n_lo, n_hi, p), s = sp.r(s0);
+            const int32_t word = sp.cell[sp.c(s0)];
+            if ((uint32_t)word & kPaired) continue;  // with its ion: no net charge
             int ci, cj, ck;
-            unpack_cell(g, sp.cell[s], ci, cj, ck);
+            unpack_cell(g, word, ci, cj, ck);
             real wx[S + 1], wy[S + 1], wz[S + 1];
             real ox = sp.ox[s], oy = DIM == 3 ? sp.oy[s] : real(0), oz = sp.oz[s];
             if (sp.dlx) {  // relative form: the offsets in the stored cell
@@ -377,7 +379,7 @@ __global__ void particle_sums_kernel(Geom g, Species<real> sp, const int *lo, co
         bucket_counts(lo, hi, t, g.cap, n_lo, n_hi, nullptr);
         const int n = n_lo + n_hi;
         for (int p = threadIdx.x; p < n; p += blockDim.x) {
-            const int64_t s = bucket_slot(t, g.cap, n_lo, n_hi, p);
+            const int64_t slot = bucket_slot(t, g.cap, n_lo, n_hi, p), s = sp.r(slot);
             const double w = (double)sp.w[s];
             // records hold u - u_drift; ions move with the drift itself
             double ux = iux, uy = iuy, uz = iuz;
@@ -388,7 +390,7 @@ __global__ void particle_sums_kernel(Geom g, Species<real> sp, const int *lo, co
             }
             const double u2 = ux * ux + uy * uy + uz * uz;
             const double ke = w * (u2 / (sqrt(1.0 + u2) + 1.0));  // gamma - 1 without cancellation
-            const bool pair = ((uint32_t)sp.cell[s] & kPaired) != 0u;
+            const bool pair = ((uint32_t)sp.cell[sp.c(slot)] & kPaired) != 0u;
             npair += pair ? 1.0 : 0.0;
             double y = ke - c0, tt = s0 + y;
             c0 = (tt - s0) - y;
