@@ -506,6 +506,22 @@ static void fill_inject_common(pic_ctx *c, InjectArgs &a)
     a.wfac = c->gam * c->vol / (double)(a.ppx * a.ppy * a.ppz);
     a.nprof = p.n_profile;
     for (int m = 0; m < 16; ++m) a.prof[m] = m < p.n_profile ? c->prof[m] : 0.0;
+    a.spx = a.hx / (double)a.ppx;
+    a.spy = a.hy / (double)a.ppy;
+    a.jx = a.jitter * a.hx;
+    a.jy = a.jitter * a.hy;
+    a.jz = a.jitter * a.hz_lab;
+    a.rhx = 1.0 / a.hx;
+    a.rhy = 1.0 / a.hy;
+    a.rhz = 1.0 / a.hz;
+    a.rgam = 1.0 / a.gam;
+    a.rlen = 1.0 / (a.z_end - a.z_start);
+    // (far from overflow and underflow: every residual of the quotients is exact)
+    a.fast = 1;
+    for (double v : {a.hx, a.hy, a.hz, a.gam, a.z_end - a.z_start})
+        if (!(v > 1e-60 && v < 1e60)) a.fast = 0;
+    for (double v : {a.z_start, a.z_end, a.Lx, a.Ly, a.Lz, a.zwin + c->Lz, c->t})
+        if (!(std::fabs(v) < 1e60)) a.fast = 0;
     a.seed = c->p.seed;
     a.zwin = c->zwin();
     a.zmin = 0.0;

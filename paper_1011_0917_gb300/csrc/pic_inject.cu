@@ -31,6 +31,20 @@ __device__ __forceinline__ double uniform01(uint64_t seed, uint64_t counter)
     return (double)(splitmix64(seed, counter) >> 11) * (1.0 / 9007199254740992.0);
 }
 
+// a / b correctly rounded, rb = 1 / b correctly rounded.  The FP64 pipe is
+// what bounds these kernels (2 lanes per SM and cycle), and b is the same for
+// a whole launch: a quotient good to one ulp from the reciprocal, then
+// Markstein's correction (P. Markstein, IBM J. Res. Dev. 34, 1990: with the
+// residual a - q b exact by a fused multiply-add and rb correctly rounded,
+// q + r rb rounds to the correctly rounded quotient), five operations in all.
+__device__ __forceinline__ double quotient(double a, double b, double rb, int fast)
+{
+    if (!fast) return a / b;
+    const double q0 = a * rb;
+    const double q = __fma_rn(__fma_rn(-b, q0, a), rb, q0);
+    return __fma_rn(__fma_rn(-b, q, a), rb, q);
+}
+
 // lab-frame density: linear up-ramp, then the cosine-series profile
 __device__ double lab_density(const InjectArgs &a, double z)
 {
@@ -41,7 +55,7 @@ __device__ double lab_density(const InjectArgs &a, double z)
     if (a.nprof > 0) {
         // cos(m pi zeta) by the recurrence cos(m t) = 2 cos t cos((m-1) t) -
         // cos((m-2) t): one cosine per point (FP64 is the slow pipe here)
-        const double zeta = (z - a.z_start) / (a.z_end - a.z_start);
+        const double zeta = quotient(z - a.z_start, a.z_end - a.z_start, a.rlen, a.fast);
         const double c1 = cos(3.141592653589793 * zeta);
         double cp = 1.0, cm = c1;
         f += a.prof[0] * c1;
@@ -57,9 +71,9 @@ __device__ double lab_density(const InjectArgs &a, double z)
 
 // position (one axis) -> cell and offset in [0,1) of the working precision
 template <typename real>
-__device__ __forceinline__ void to_cell(double x, double h, int n, bool periodic, int &c, real &off)
+__device__ __forceinline__ void to_cell(double x, double h, double rh, int fast, int n, bool periodic, int &c, real &off)
 {
-    const double xi = x / h;
+    const double xi = quotient(x, h, rh, fast);
     double f = floor(xi);
     c = (int)f;
     double o = xi - f;
@@ -103,6 +117,7 @@ __device__ __forceinline__ void inject_body(const InjectArgs &a, const int64_t b
     // the step's times and lattice band (from device memory in a captured step)
     const double t = a.scal ? a.scal->t : a.t, t1 = a.scal ? a.scal->t1 : a.t1;
     const int64_t m_lo = a.scal ? a.scal->m_lo : a.m_lo, m_hi = a.scal ? a.scal->m_hi : a.m_hi;
+    const double bt = a.beta * t, bt1 = a.beta * t1;
     const int64_t total = (m_hi - m_lo) * a.NY * a.NX;
     const int64_t nround = (total + 31) / 32 * 32;
     const int64_t stride = nb * blockDim.x;
@@ -119,39 +134,38 @@ __device__ __forceinline__ void inject_body(const InjectArgs &a, const int64_t b
             const int64_t m = m_lo + r / a.NY;
             L = (m * a.NY + iy) * a.NX + ix;
             const uint64_t c0 = 3ull * (uint64_t)L;
-            double x = ((double)ix + 0.5) * (a.hx / (double)a.ppx) +
-                       (a.jitter * a.hx) * (2.0 * uniform01(a.seed, c0) - 1.0);
-            if (x < 0.0) x += a.Lx;
-            if (x >= a.Lx) x -= a.Lx;
-            double y = 0.0;
-            if (dim3) {
-                y = ((double)iy + 0.5) * (a.hy / (double)a.ppy) +
-                    (a.jitter * a.hy) * (2.0 * uniform01(a.seed, c0 + 1ull) - 1.0);
-                if (y < 0.0) y += a.Ly;
-                if (y >= a.Ly) y -= a.Ly;
+            // z first: most planes of a step's band hold no point that
+            // crosses now, and their points are done here
+            const double zlab = a.z_start + ((double)m + 0.5) * a.dzl + a.jz * (2.0 * uniform01(a.seed, c0 + 2ull) - 1.0);
+            // simulation-frame positions relative to the (moving) window
+            const double zg = quotient(zlab, a.gam, a.rgam, a.fast);
+            bool take;
+            double zb;
+            if (a.mode == 0) {
+                zb = zg - bt - a.zwin;
+                take = zb >= a.zmin && zb < a.Lz;
+            } else {
+                const double zb0 = zg - bt - a.zwin;
+                zb = zg - bt1 - a.zwin;
+                take = zb0 >= a.Lz && zb < a.Lz;
             }
-            const double zlab = a.z_start + ((double)m + 0.5) * a.dzl +
-                                (a.jitter * a.hz_lab) * (2.0 * uniform01(a.seed, c0 + 2ull) - 1.0);
-            zeta = (zlab - a.z_start) / (a.z_end - a.z_start);
-            const double n = lab_density(a, zlab);
-            if (n > 0.0) {
-                bool take;
-                double zb;
-                // simulation-frame positions relative to the (moving) window
-                if (a.mode == 0) {
-                    zb = zlab / a.gam - a.beta * t - a.zwin;
-                    take = zb >= a.zmin && zb < a.Lz;
-                } else {
-                    const double zb0 = zlab / a.gam - a.beta * t - a.zwin;
-                    zb = zlab / a.gam - a.beta * t1 - a.zwin;
-                    take = zb0 >= a.Lz && zb < a.Lz;
-                }
-                if (take) {
-                    to_cell<real>(x, a.hx, a.g.nx, true, ci, ox);
-                    if (dim3) to_cell<real>(y, a.hy, a.g.ny, true, cj, oy);
-                    to_cell<real>(zb, a.hz, a.g.nz, a.g.bc_z == 0, ck, oz);
+            if (take) {
+                const double n = lab_density(a, zlab);
+                if (n > 0.0) {
+                    double x = ((double)ix + 0.5) * a.spx + a.jx * (2.0 * uniform01(a.seed, c0) - 1.0);
+                    if (x < 0.0) x += a.Lx;
+                    if (x >= a.Lx) x -= a.Lx;
+                    to_cell<real>(x, a.hx, a.rhx, a.fast, a.g.nx, true, ci, ox);
+                    if (dim3) {
+                        double y = ((double)iy + 0.5) * a.spy + a.jy * (2.0 * uniform01(a.seed, c0 + 1ull) - 1.0);
+                        if (y < 0.0) y += a.Ly;
+                        if (y >= a.Ly) y -= a.Ly;
+                        to_cell<real>(y, a.hy, a.rhy, a.fast, a.g.ny, true, cj, oy);
+                    }
+                    to_cell<real>(zb, a.hz, a.rhz, a.fast, a.g.nz, a.g.bc_z == 0, ck, oz);
                     wr = (real)(n * a.wfac);
                     dest = tile_of(a.g, ci, cj, ck);
+                    if (a.flat_base >= 0) zeta = quotient(zlab - a.z_start, a.z_end - a.z_start, a.rlen, a.fast);
                 }
             }
         }

@@ -499,6 +499,11 @@ struct InjectArgs {      // lattice load / boosted injection, FP64
     double z_start, z_end, ramp, ne, jitter, dzl, hz_lab, wfac;
     int nprof;
     double prof[16];
+    // of the launch, rounded as the kernel's expressions would: the lattice
+    // spacings across, the jitters, and the reciprocals of the divisors (with
+    // fast set: see quotient)
+    double spx, spy, jx, jy, jz, rhx, rhy, rhz, rgam, rlen;
+    int fast;
     uint64_t seed;
     int mode;           // 0: in [zmin, Lz) at t; 1: crossing z = Lz during (t, t1]
     double t, t1;
