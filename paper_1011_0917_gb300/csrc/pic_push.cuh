@@ -121,17 +121,72 @@ __device__ __forceinline__ void sh_acc2(int *p, f32x2 a, f32x2 b, f32x2 lo_scale
     sh_add(p + LOFF + STRIDE, (int)(unsigned)(l >> 32) - kRoundMagicBits);
 }
 
-// FP64 contributions into the same fixed-point words (records in relative
-// form): h and the remainder's 2^K multiple rounded from the FP64 product
-template <int LOFF>
-__device__ __forceinline__ void sh_acc(int *p, double a, double b, double lo_scale)
+// An unevaluated sum h + l of two FP32 values, |l| <= ulp(h) / 2: about 48
+// bits, from the error-free sum and product (Knuth, TAOCP 2, 4.2.2; Dekker,
+// Numer. Math. 18, 1971, with a fused multiply-add for the product's error).
+// The currents of records in relative form need their exact positions and far
+// more than FP32's bits (see rel_actual), and end in fixed-point words that
+// carry at most 43 bits; FP64 arithmetic gives 2 lanes per SM and cycle here,
+// FP32 128, of which one of these operations takes 7 to 11.
+struct ff {
+    float h, l;
+    __device__ __forceinline__ ff() {}
+    __device__ __forceinline__ ff(float x) : h(x), l(0.0f) {}
+    __device__ __forceinline__ ff(int x) : h((float)x), l(0.0f) {}
+    __device__ __forceinline__ ff(double x) : h((float)x), l((float)(x - (double)(float)x)) {}
+    __device__ __forceinline__ ff(float x, float y) : h(x), l(y) {}
+};
+__device__ __forceinline__ ff two_sum(float a, float b)
 {
-    const double v = a * b;
-    const double hd = rint(v);
-    const int h = (int)hd;
-    const int l = (int)rint((v - hd) * lo_scale);
-    if (h != 0) atomicAdd(p, h);
-    if (l != 0) atomicAdd(p + LOFF, l);
+    const float s = __fadd_rn(a, b), z = __fsub_rn(s, a);
+    return ff(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z)));
+}
+// |a| >= |b| or a = 0
+__device__ __forceinline__ ff quick_sum(float a, float b)
+{
+    const float s = __fadd_rn(a, b);
+    return ff(s, __fsub_rn(b, __fsub_rn(s, a)));
+}
+__device__ __forceinline__ ff operator+(ff a, ff b)
+{
+    const ff s = two_sum(a.h, b.h);
+    return quick_sum(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ ff operator-(ff a) { return ff(-a.h, -a.l); }
+__device__ __forceinline__ ff operator-(ff a, ff b) { return a + -b; }
+__device__ __forceinline__ ff operator*(ff a, ff b)
+{
+    const float p = __fmul_rn(a.h, b.h);
+    float e = __fmaf_rn(a.h, b.h, -p);
+    e = __fmaf_rn(a.h, b.l, e);
+    e = __fmaf_rn(a.l, b.h, e);
+    return quick_sum(p, e);
+}
+__device__ __forceinline__ ff &operator+=(ff &a, ff b)
+{
+    a = a + b;
+    return a;
+}
+__device__ __forceinline__ bool operator==(ff a, ff b) { return a.h == b.h && a.l == b.l; }
+// the exact floor (the low word decides where the high one is an integer)
+__device__ __forceinline__ float floor_ff(ff a)
+{
+    const float f = floorf(a.h);
+    return a.h == f && a.l < 0.0f ? f - 1.0f : f;
+}
+
+// contributions of records in relative form into the same fixed-point words
+template <int LOFF>
+__device__ __forceinline__ void sh_acc(int *p, ff a, ff b, ff lo_scale)
+{
+    const float v = __fmul_rn(a.h, b.h);
+    float e = __fmaf_rn(a.h, b.h, -v);
+    e = __fmaf_rn(a.h, b.l, e);
+    e = __fmaf_rn(a.l, b.h, e);
+    const float t = __fadd_rn(v, kRoundMagic);
+    const float r = __fadd_rn(__fsub_rn(v, __fsub_rn(t, kRoundMagic)), e);
+    sh_add(p, __float_as_int(t) - kRoundMagicBits);
+    sh_add(p + LOFF, __float_as_int(__fmaf_rn(r, lo_scale.h, kRoundMagic)) - kRoundMagicBits);
 }
 
 template <int LOFF>
@@ -415,7 +470,7 @@ __device__ __forceinline__ void deposit_w(accT *sJ, const real *S0x, const real 
                                           real fx, real fy, real fz, real fyv, real los)
 {
     constexpr int LOFF = 3 * QN;  // "lo" words follow the three components' "hi" words
-    constexpr real half = real(0.5), third = real(1) / real(3);
+    const real half = real(0.5), third = real(1.0 / 3.0);
     auto *Jx = sJ, *Jy = sJ + QN, *Jz = sJ + 2 * QN;
     if constexpr (sizeof(real) == 4) {
         deposit_w2<DIM, QX, QY, QN, WX, WY, WZ>(sJ, S0x, DSx, S0y, DSy, S0z, DSz, ax, ay, az, fx, fy, fz, fyv, los);
@@ -552,6 +607,55 @@ __device__ __forceinline__ void deposit_sel(unsigned sel, accT *sJ, const real *
         }
     }
 #undef PIC_DEP
+}
+
+// Esirkepov's window along one axis for records in relative form: both ends
+// in ff or FP64, each within a cell of [0, 1) (esirk_axis_g, whose FP64 form
+// the debug path takes).
+template <int S>
+__device__ __forceinline__ float spline_ff(ff p, ff w[S + 1])
+{
+    if (S == 1) {
+        const float f = floor_ff(p);
+        const ff d = p - ff(f);
+        w[0] = ff(1.0f) - d;
+        w[1] = d;
+        return f;
+    }
+    const float c = floor_ff(p + ff(0.5f));
+    const ff d = p - ff(c), a = ff(0.5f) - d, b = ff(0.5f) + d;
+    w[0] = ff(0.5f) * (a * a);
+    w[1] = ff(0.75f) - d * d;
+    w[2] = ff(0.5f) * (b * b);
+    return c - 1.0f;
+}
+template <int S>
+__device__ __forceinline__ int esirk_rel(ff x0, ff x1, ff S0[S + 2], ff DS[S + 2], bool &crossed)
+{
+    ff w0[S + 1], w1[S + 1];
+    const float b0 = spline_ff<S>(x0, w0), b1 = spline_ff<S>(x1, w1);
+    const bool s0 = b0 > b1, s1 = b1 > b0;  // which support starts a node above the window
+    crossed = b0 != b1;
+#pragma unroll
+    for (int q = 0; q < S + 2; ++q) {
+        const ff lo0 = q <= S ? w0[q <= S ? q : S] : ff(0.0f), hi0 = q >= 1 ? w0[q >= 1 ? q - 1 : 0] : ff(0.0f);
+        const ff lo1 = q <= S ? w1[q <= S ? q : S] : ff(0.0f), hi1 = q >= 1 ? w1[q >= 1 ? q - 1 : 0] : ff(0.0f);
+        const ff v1 = ff(s1 ? hi1.h : lo1.h, s1 ? hi1.l : lo1.l);
+        S0[q] = ff(s0 ? hi0.h : lo0.h, s0 ? hi0.l : lo0.l);
+        DS[q] = v1 - S0[q];
+    }
+    return (int)fminf(b0, b1);
+}
+template <int S>
+__device__ __forceinline__ int esirk_rel(double x0, double x1, double S0[S + 2], double DS[S + 2], bool &crossed)
+{
+    return esirk_axis_g<S>(x0, x1, S0, DS, crossed);
+}
+// a position in the arithmetic of the deposit: r + (o + dl), exact
+template <typename T> __device__ __forceinline__ T rel_pos(int r, double o, double dl) { return (T)r + (o + dl); }
+template <typename T> __device__ __forceinline__ T rel_pos(int r, float o, float dl)
+{
+    return T(r) + two_sum(o, dl);
 }
 
 // One axis of the CIC window from the in-cell offset o, the offset d in the
@@ -761,10 +865,16 @@ __device__ __forceinline__ void ion_deposit(accT *Jz, ar z0, ar z1, ar ox, ar oy
     constexpr int JL = S;
     ar S0z[S + 2], DSz[S + 2], wx[S + 1], wy[S + 1];
     bool crossed;
-    const int az = esirk_axis_c<S>(z0, z1, S0z, DSz, crossed) + lk + JL;
-    const int bx = offset_weights<S>(ox, wx) + li + JL;
-    int by = 0;
-    if (DIM == 3) by = offset_weights<S>(oy, wy) + lj + JL;
+    int az, bx, by = 0;
+    if constexpr (std::is_same<ar, ff>::value) {
+        az = esirk_rel<S>(z0, z1, S0z, DSz, crossed) + lk + JL;
+        bx = (int)spline_ff<S>(ox, wx) + li + JL;
+        if (DIM == 3) by = (int)spline_ff<S>(oy, wy) + lj + JL;
+    } else {
+        az = esirk_axis_c<S>(z0, z1, S0z, DSz, crossed) + lk + JL;
+        bx = offset_weights<S>(ox, wx) + li + JL;
+        if (DIM == 3) by = offset_weights<S>(oy, wy) + lj + JL;
+    }
     ar Pz[S + 2];
     ar run = 0;
 #pragma unroll
@@ -803,8 +913,8 @@ __device__ __forceinline__ void ion_deposit(accT *Jz, ar z0, ar z1, ar ox, ar oy
 // The ions of tile t (all threads of the CTA call it): their Jz into the
 // current tile at Jz (the "hi" words; the "lo" words LOFF further), records
 // into the output side.  wbuf: the warp's buffer.  REL: the tile's electrons
-// are in relative form; the ions' currents are then formed in FP64 from their
-// stored positions (the end of one step's path is exactly the start of the
+// are in relative form; the ions' currents are then formed in their arithmetic
+// (ff) from their stored positions (the end of one step's path is exactly the start of the
 // next one's).  Returns false (nothing done) for an empty bucket.  The loop
 // runs all lanes of a warp (as the electrons', see push_tile).
 template <typename real, int DIM, int S, int TX, int TY, int TZ, int LOFF, bool REL>
@@ -817,6 +927,7 @@ __device__ __forceinline__ bool ions_of_tile(const Geom &g, const IonSide<real> 
     constexpr int QX = TX + JL + JH, QY = DIM == 3 ? TY + JL + JH : 1;
     using acc_t = typename Acc<real>::type;
     using R = Rec<real, DIM, false, false>;
+    using rel_t = typename std::conditional<sizeof(real) == 4, ff, double>::type;
     constexpr int ES = (int)sizeof(real), kBlock = BlockOf<real, DIM>::value;
     int n_lo, n_hi;
     bucket_counts(is.in_lo, is.in_hi, t, g.cap, n_lo, n_hi, err);
@@ -898,9 +1009,10 @@ __device__ __forceinline__ bool ions_of_tile(const Geom &g, const IonSide<real> 
         oz = z1 < real(0) ? (sz ? up : real(0)) : z1;
         if (valid) {
             if (REL)  // from the stored position to the stored position
-                ion_deposit<double, acc_t, DIM, S, QX, QY, LOFF>(
-                    Jz, (double)z0, (double)sz + (double)oz, (double)ox, (double)oy, li, lj, lk,
-                    (double)is.jfac_z * (double)w * (double)scale_z, (double)lo_scale);
+                ion_deposit<rel_t, acc_t, DIM, S, QX, QY, LOFF>(Jz, rel_t(z0), rel_pos<rel_t>(sz, oz, real(0)), rel_t(ox),
+                                                                rel_t(oy), li, lj, lk,
+                                                                rel_t(is.jfac_z) * rel_t(w) * rel_t(scale_z),
+                                                                rel_t(lo_scale));
             else
                 ion_deposit<real, acc_t, DIM, S, QX, QY, LOFF>(Jz, z0, z1, ox, oy, li, lj, lk, is.jfac_z * w * scale_z,
                                                                lo_scale);
@@ -963,8 +1075,8 @@ __device__ __forceinline__ real rel_step(real dl, real d, int &fold)
 }
 
 // REL: electron records in relative form (rel_actual): the gather uses the
-// offsets in the stored cell, the current is deposited in FP64 from the exact
-// positions reference + departure.
+// offsets in the stored cell, the current is deposited in ff arithmetic from
+// the exact positions reference + departure.
 //
 // The loop is bound by issue slots and the latency they hide, so it runs all
 // 32 lanes of a warp without per-lane branches: lanes without a record (the
@@ -993,8 +1105,9 @@ __device__ __forceinline__ void push_tile(const PushArgs<real> &a, const int64_t
     using R = Rec<real, DIM, true, REL>;
     using RI = Rec<real, DIM, false, false>;
     constexpr int ES = (int)sizeof(real);
-    // arithmetic of the deposit: FP64 for records in relative form
-    using dep_t = typename std::conditional<REL, double, real>::type;
+    // arithmetic of the deposit: pairs of FP32 words for records in relative
+    // form (FP64 in the debug path)
+    using dep_t = typename std::conditional<REL && sizeof(real) == 4, ff, real>::type;
     unsigned char *wbuf = smem_raw + (threadIdx.x >> 5) * warp_bytes<R>();
     unsigned char *q = wbuf + R::RB;
     int *qmove = reinterpret_cast<int *>(q + R::RB), *qslot = qmove + 32;
@@ -1186,27 +1299,25 @@ __device__ __forceinline__ void push_tile(const PushArgs<real> &a, const int64_t
             }
         }
         // new offsets nox .. and the new cell relative to the old (mx ..);
-        // relative form: new departures, and the exact (FP64) start and end
-        // of the path relative to the old cell; else the end of the path and
-        // its cell (fx ..)
+        // relative form: new departures, and the shift of the reference cell
+        // at the path's end (rx1 ..), relative to the old cell; else the end
+        // of the path and its cell (fx ..)
         real nox, noy = 0, noz, dlx1 = 0, dly1 = 0, dlz1 = 0;
         real x1 = 0, y1 = 0, z1 = 0, fx = 0, fy = 0, fz = 0;
         int mx, my = 0, mz;
-        double X0 = 0, X1 = 0, Y0 = 0, Y1 = 0, Z0 = 0, Z1 = 0;
+        int rx1 = 0, ry1 = 0, rz1 = 0;
         if (REL) {
             // across z the reference stays, the departure moves
             int f, r1;
             dlx1 = rel_step(dlx, dx, f);
             (void)rel_actual(orx, dlx1, r1);
             mx = rx + f - r1;
-            X0 = (double)rx + ((double)orx + (double)dlx);
-            X1 = (double)(rx + f) + ((double)orx + (double)dlx1);
+            rx1 = rx + f;
             if (DIM == 3) {
                 dly1 = rel_step(dly, dy, f);
                 (void)rel_actual(ory, dly1, r1);
                 my = ry + f - r1;
-                Y0 = (double)ry + ((double)ory + (double)dly);
-                Y1 = (double)(ry + f) + ((double)ory + (double)dly1);
+                ry1 = ry + f;
             }
             // along z the reference moves exactly like a drifting ion
             // (same rounding, same cell changes)
@@ -1223,8 +1334,7 @@ __device__ __forceinline__ void push_tile(const PushArgs<real> &a, const int64_t
             dlz1 = rel_step(dlz, ddz, f);
             (void)rel_actual(sref, dlz1, r1);
             mz = rz + sr + f - r1;
-            Z0 = (double)rz + ((double)orz + (double)dlz);
-            Z1 = (double)(rz + sr + f) + ((double)sref + (double)dlz1);
+            rz1 = rz + sr + f;
             nox = orx;  // x, y references do not move
             noy = ory;
             noz = sref;
@@ -1318,10 +1428,10 @@ __device__ __forceinline__ void push_tile(const PushArgs<real> &a, const int64_t
         deposited = true;
         // (the fixed-point factors are read from the parameters at each use:
         // held in registers they would cost spills here)
-        const dep_t jx = (dep_t)a.jfac[0] * (dep_t)w * (dep_t)a.fx_scale[0];
-        const dep_t jy = (dep_t)a.jfac[1] * (dep_t)w * (dep_t)a.fx_scale[1];
-        const dep_t jz = (dep_t)a.jfac[2] * (dep_t)w * (dep_t)a.fx_scale[2];
-        const dep_t jyv = (dep_t)a.jyfac * (dep_t)w * (dep_t)vy * (dep_t)a.fx_scale[1];
+        const dep_t jx = dep_t(a.jfac[0]) * dep_t(w) * dep_t(a.fx_scale[0]);
+        const dep_t jy = dep_t(a.jfac[1]) * dep_t(w) * dep_t(a.fx_scale[1]);
+        const dep_t jz = dep_t(a.jfac[2]) * dep_t(w) * dep_t(a.fx_scale[2]);
+        const dep_t jyv = dep_t(a.jyfac) * dep_t(w) * dep_t(vy) * dep_t(a.fx_scale[1]);
         if constexpr (S == 1 && !REL && ES == 4) {
             const bool z_only = DIM == 3 && __all_sync(kAll, !dep || (x1 == ox && y1 == oy));
             const unsigned sel = (__any_sync(kAll, dep && fx != 0.0f) ? 4u : 0u) |
@@ -1335,10 +1445,14 @@ __device__ __forceinline__ void push_tile(const PushArgs<real> &a, const int64_t
             int ax = 0, ay = 0, az = 0;
             bool cx = false, cy = false, cz = false;
             if (dep) {
-                if (REL) {
-                    ax = esirk_axis_g<S, dep_t>((dep_t)X0, (dep_t)X1, S0x, DSx, cx) + li + JL;
-                    az = esirk_axis_g<S, dep_t>((dep_t)Z0, (dep_t)Z1, S0z, DSz, cz) + lk + JL;
-                    if (DIM == 3) ay = esirk_axis_g<S, dep_t>((dep_t)Y0, (dep_t)Y1, S0y, DSy, cy) + lj + JL;
+                if constexpr (REL) {
+                    ax = esirk_rel<S>(rel_pos<dep_t>(rx, orx, dlx), rel_pos<dep_t>(rx1, orx, dlx1), S0x, DSx, cx) + li +
+                         JL;
+                    az = esirk_rel<S>(rel_pos<dep_t>(rz, orz, dlz), rel_pos<dep_t>(rz1, noz, dlz1), S0z, DSz, cz) + lk +
+                         JL;
+                    if (DIM == 3)
+                        ay = esirk_rel<S>(rel_pos<dep_t>(ry, ory, dly), rel_pos<dep_t>(ry1, ory, dly1), S0y, DSy, cy) +
+                             lj + JL;
                 } else {
                     ax = esirk_axis_c<S, dep_t>(ox, x1, S0x, DSx, cx) + li + JL;
                     az = esirk_axis_c<S, dep_t>(oz, z1, S0z, DSz, cz) + lk + JL;
@@ -1349,7 +1463,8 @@ __device__ __forceinline__ void push_tile(const PushArgs<real> &a, const int64_t
                                  (__any_sync(kAll, cz) ? 1u : 0u);
             // 3D: no lane moved in x or y (e.g. plasma the laser has not reached)
             const bool z_only =
-                DIM == 3 && __all_sync(kAll, !dep || (REL ? (X1 == X0 && Y1 == Y0) : (x1 == ox && y1 == oy)));
+                DIM == 3 && __all_sync(kAll, !dep || (REL ? (rx1 == rx && dlx1 == dlx && ry1 == ry && dly1 == dly)
+                                                         : (x1 == ox && y1 == oy)));
             if (dep) {
                 if (z_only) {
                     if (sel & 1u)
