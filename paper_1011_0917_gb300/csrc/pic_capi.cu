@@ -417,7 +417,7 @@ extern "C" pic_status pic_init_grid(const pic_grid_params *p, pic_ctx **out)
     c->off_offsets = o;
     o += align_up(sizeof(int64_t) * (size_t)g.ntiles);
     c->off_partials = o;
-    o += align_up(sizeof(double) * 3 * kPartialBlocks);
+    o += align_up(sizeof(double) * 9 * kPartialBlocks);
     c->off_err = o;
     o += kAlign;
     c->off_eb = o;
@@ -1957,35 +1957,45 @@ static double kahan_sum(const double *v, size_t n, size_t stride)
     return s;
 }
 
+// the sums of fields and species: all kernels, then one copy and one wait
 template <typename real>
 static pic_status diagnostics_t(pic_ctx *c, pic_diag *out)
 {
     double *part = reinterpret_cast<double *>(c->scratch + c->off_partials);
-    std::vector<double> h(3 * kPartialBlocks);
+    const int nsp = c->ions_species ? 2 : 1;
     real *F[9];
     for (int q = 0; q < 9; ++q) F[q] = (real *)field_ptr(c, q);
-    launch_field_sums<real>(c->g, F, part, kPartialBlocks, c->stream);
+    const int nf = launch_field_sums<real>(c->g, F, part, kPartialBlocks, c->stream);
+    int nb[2] = {0, 0};
+    size_t used = (size_t)nf;
+    for (int sp = 0; sp < nsp; ++sp) {
+        nb[sp] = launch_particle_sums<real>(c->g, species_view<real>(c, sp, c->cur[sp]), counts(c, sp, c->cur[sp], 0),
+                                            counts(c, sp, c->cur[sp], 1), sp == 0 ? -1.0 : 1.0, drift_u<real>(c),
+                                            part + used, kPartialBlocks, c->stream);
+        used += (size_t)4 * nb[sp];
+    }
     CUDA_TRY(c, cudaGetLastError());
-    CUDA_TRY(c, cudaMemcpyAsync(h.data(), part, sizeof(double) * kPartialBlocks, cudaMemcpyDeviceToHost, c->stream));
+    std::vector<double> h(used);
+    CUDA_TRY(c, cudaMemcpyAsync(h.data(), part, sizeof(double) * used, cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-    out->field_energy = 0.5 * c->vol * kahan_sum(h.data(), kPartialBlocks, 1);
+    out->field_energy = 0.5 * c->vol * kahan_sum(h.data(), (size_t)nf, 1);
     out->kinetic_energy = 0;
     out->charge = 0;
-    const real u_drift[3] = {0, 0, drift_u<real>(c)};
-    for (int sp = 0; sp < (c->ions_species ? 2 : 1); ++sp) {
-        launch_particle_sums<real>(c->g, species_view<real>(c, sp, c->cur[sp]), counts(c, sp, c->cur[sp], 0),
-                                   counts(c, sp, c->cur[sp], 1), sp == 0 ? -1.0 : 1.0, u_drift, part, kPartialBlocks,
-                                   c->stream);
-        CUDA_TRY(c, cudaGetLastError());
-        CUDA_TRY(c, cudaMemcpyAsync(h.data(), part, sizeof(double) * 3 * kPartialBlocks, cudaMemcpyDeviceToHost, c->stream));
-        CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-        if (sp == 0) {
-            out->kinetic_energy = kahan_sum(h.data(), kPartialBlocks, 3);
-            double np = 0;
-            for (int b = 0; b < kPartialBlocks; ++b) np += h[3 * b + 2];
-            out->n_paired = (int64_t)np;
+    const double *p = h.data() + nf;
+    for (int sp = 0; sp < nsp; ++sp) {
+        double pairs = 0, records = 0;
+        for (int b = 0; b < nb[sp]; ++b) {
+            if (p[4 * b + 3] < 0) return fail(c, PIC_ERR_CAPACITY, "a tile bucket overflowed (raise slots_per_cell)");
+            pairs += p[4 * b + 2];
+            records += p[4 * b + 3];
         }
-        out->charge += kahan_sum(h.data() + 1, kPartialBlocks, 3);
+        out->n_particles[sp] = (int64_t)records;
+        if (sp == 0) {
+            out->kinetic_energy = kahan_sum(p, (size_t)nb[sp], 4);
+            out->n_paired = (int64_t)pairs;
+        }
+        out->charge += kahan_sum(p + 1, (size_t)nb[sp], 4);
+        p += 4 * nb[sp];
     }
     return PIC_OK;
 }
@@ -1998,14 +2008,6 @@ extern "C" pic_status pic_get_diagnostics(pic_ctx *c, pic_diag *out)
     out->t = c->t;
     out->step = c->step;
     out->z_window = c->zwin();
-    for (int sp = 0; sp < 2; ++sp) {
-        if (sp == 1 && !c->ions_species) break;
-        std::vector<int64_t> off;
-        int64_t n = 0;
-        pic_status s = tile_offsets(c, sp, off, n);
-        if (s != PIC_OK) return s;
-        out->n_particles[sp] = n;
-    }
     pic_status s = c->es == 4 ? diagnostics_t<float>(c, out) : diagnostics_t<double>(c, out);
     if (s == PIC_OK) out->n_particles[1] += out->n_paired;
     return s;

@@ -401,6 +401,63 @@ __device__ __forceinline__ real drift_velocity(const Drift<real> &d, real dux, r
     return (duz * (real(2) + E) - d.U * p2) * (ig * d.ig * is);
 }
 
+// Sums of many values of the working precision in FP64, compensated.  The
+// FP64 pipe takes 2 lanes per SM and cycle, so an FP32 value is not converted
+// and added by itself: up to kSumRun of them go into an unevaluated sum of
+// three FP32 words by error-free two-sums (Knuth, TAOCP 2, 4.2.2), exact to
+// far below FP64's last bit, and the three into an FP64 Kahan sum.  (With two
+// words the totals were off by 4e-16 to 9e-16 of the sum, all to one side;
+// FP64 Kahan sums of every value by 2e-16.)  FP64 values are added by Kahan
+// directly.
+constexpr int kSumRun = 32;
+struct Kahan {
+    double s = 0, c = 0;
+    __device__ __forceinline__ void add(double v)
+    {
+        const double y = v - c, t = s + y;
+        c = (t - s) - y;
+        s = t;
+    }
+    __device__ __forceinline__ double value() const { return s - c; }
+};
+template <typename real> struct RunSum {
+    Kahan k;
+    __device__ __forceinline__ void add(double v) { k.add(v); }
+    __device__ __forceinline__ void add_square(double v) { k.add(v * v); }
+    __device__ __forceinline__ void flush() {}
+};
+template <> struct RunSum<float> {
+    Kahan k;
+    float h = 0, l = 0, m = 0;
+    // a += b, the rounding error returned
+    static __device__ __forceinline__ float add_to(float &a, float b)
+    {
+        const float t = __fadd_rn(a, b), z = __fsub_rn(t, a);
+        const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(t, z)), __fsub_rn(b, z));
+        a = t;
+        return e;
+    }
+    __device__ __forceinline__ void add(float v) { m = __fadd_rn(m, add_to(l, add_to(h, v))); }
+    // v^2 exactly: its rounded product and the product's error (in FP64
+    // where either might leave the FP32 range)
+    __device__ __forceinline__ void add_square(float v)
+    {
+        const float a = fabsf(v);
+        if (!(a > 1e-12f && a < 1e15f) && a != 0.0f) {
+            k.add((double)v * (double)v);
+            return;
+        }
+        const float p = __fmul_rn(v, v);
+        m = __fadd_rn(m, add_to(l, __fmaf_rn(v, v, -p)));
+        add(p);
+    }
+    __device__ __forceinline__ void flush()
+    {
+        k.add((double)h + ((double)l + (double)m));
+        h = l = m = 0.0f;
+    }
+};
+
 // largest value below one, for offsets that round up to 1
 template <typename real> __host__ __device__ inline real below_one();
 template <> __host__ __device__ inline float below_one<float>() { return 0.99999994f; }
@@ -698,8 +755,8 @@ template <typename real>
 void launch_rho(const Geom &g, const Species<real> &sp, const int *lo, const int *hi, real qfac, real *rho,
                 cudaStream_t s);
 template <typename real>
-void launch_particle_sums(const Geom &g, const Species<real> &sp, const int *lo, const int *hi, double q,
-                          const real u_drift[3], double *partials, int nblocks, cudaStream_t s);
+int launch_particle_sums(const Geom &g, const Species<real> &sp, const int *lo, const int *hi, double q,
+                          real u_drift, double *partials, int max_blocks, cudaStream_t s);
 void launch_inject(const InjectArgs &a, cudaStream_t s);
 template <typename real>
 void launch_btd(const BtdArgs<real> &a, cudaStream_t s);
@@ -734,7 +791,7 @@ template <typename real>
 void launch_antenna(const Geom &g, real *J, int pol, int ka, double j0, double hx, double hy,
                     double xc, double yc, double waist, cudaStream_t s, const double *j0p = nullptr);
 template <typename real>
-void launch_field_sums(const Geom &g, real *const F[9], double *partials, int nblocks,
+int launch_field_sums(const Geom &g, real *const F[9], double *partials, int nblocks,
                        cudaStream_t s);
 // adjoint: flat forward steps (electrons, and the slots' ions) and their transposes
 template <typename real> void launch_adj_push(const AdjArgs<real> &a, cudaStream_t s);

@@ -4,6 +4,9 @@
 // density and particle sums.
 #include "pic_push.cuh"
 
+#include <algorithm>
+#include <cmath>
+
 namespace pic {
 
 template <typename real, int DIM, int S, int TX, int TY, int TZ, bool REL>
@@ -365,68 +368,93 @@ void launch_rho(const Geom &g, const Species<real> &sp, const int *lo, const int
 
 // -------------------------------------------------------- particle sums
 
-// Kahan-compensated FP64 partial sums per block: [0] sum w (gamma-1),
-// [1] sum q w (a paired electron and its ion carry no net charge), [2] the
-// number of paired electrons.  The host adds the block partials, also with
-// compensation.
+// Compensated FP64 partial sums per block: [0] sum w (gamma-1), [1] sum q w (a
+// paired electron and its ion carry no net charge), [2] the number of paired
+// electrons, [3] the number of records (negative: a bucket overflowed).  The
+// host adds the block partials, also with compensation.
+// Records at rest relative to the drift (all ions; the electrons no field has
+// reached, most of a boosted plasma) share one gamma - 1, rest_ke: only their
+// weights are summed.  (256 x 8192 cells, 8.4M electrons, 6% of them moving: 324 us
+// per species with the FP64 kinetic energy of every record.)
 template <typename real>
-__global__ void particle_sums_kernel(Geom g, Species<real> sp, const int *lo, const int *hi, double q,
-                                     double iux, double iuy, double iuz, double *partials)
+__global__ void particle_sums_kernel(Geom g, Species<real> sp, const int *lo, const int *hi, double q, double iuz,
+                                     double rest_ke, double *partials)
 {
-    double s0 = 0, c0 = 0, s1 = 0, c1 = 0, npair = 0;
+    RunSum<real> rest, charge;
+    Kahan moving;
+    unsigned npair = 0;
+    int run = 0;
+    double records = 0;
+    unsigned overflow = 0;
     for (int64_t t = blockIdx.x; t < g.ntiles; t += gridDim.x) {
         int n_lo, n_hi;
         bucket_counts(lo, hi, t, g.cap, n_lo, n_hi, nullptr);
+        if (hi[t] > n_hi) overflow = 1;  // (clamped: the runs meet)
         const int n = n_lo + n_hi;
+        if (threadIdx.x == 0) records += n;
         for (int p = threadIdx.x; p < n; p += blockDim.x) {
             const int64_t slot = bucket_slot(t, g.cap, n_lo, n_hi, p), s = sp.r(slot);
-            const double w = (double)sp.w[s];
-            // records hold u - u_drift; ions move with the drift itself
-            double ux = iux, uy = iuy, uz = iuz;
-            if (sp.ux) {
-                ux += (double)sp.ux[s];
-                uy += (double)sp.uy[s];
-                uz += (double)sp.uz[s];
-            }
-            const double u2 = ux * ux + uy * uy + uz * uz;
-            const double ke = w * (u2 / (sqrt(1.0 + u2) + 1.0));  // gamma - 1 without cancellation
+            const real w = sp.w[s];
             const bool pair = ((uint32_t)sp.cell[sp.c(slot)] & kPaired) != 0u;
-            npair += pair ? 1.0 : 0.0;
-            double y = ke - c0, tt = s0 + y;
-            c0 = (tt - s0) - y;
-            s0 = tt;
-            y = (pair ? 0.0 : q * w) - c1;
-            tt = s1 + y;
-            c1 = (tt - s1) - y;
-            s1 = tt;
+            real ux = 0, uy = 0, uz = 0;  // records hold u - u_drift
+            if (sp.ux) {
+                ux = sp.ux[s];
+                uy = sp.uy[s];
+                uz = sp.uz[s];
+            }
+            npair += pair ? 1u : 0u;
+            if (!pair) charge.add(w);
+            if (ux == real(0) && uy == real(0) && uz == real(0)) {
+                rest.add(w);
+            } else {
+                const double vx = (double)ux, vy = (double)uy, vz = iuz + (double)uz;
+                const double u2 = vx * vx + vy * vy + vz * vz;
+                moving.add((double)w * (u2 / (sqrt(1.0 + u2) + 1.0)));  // gamma - 1 without cancellation
+            }
+            if (++run == kSumRun) {
+                rest.flush();
+                charge.flush();
+                run = 0;
+            }
         }
     }
-    __shared__ double red[3][256];
-    red[0][threadIdx.x] = s0 - c0;
-    red[1][threadIdx.x] = s1 - c1;
-    red[2][threadIdx.x] = npair;
+    rest.flush();
+    charge.flush();
+    __shared__ double red[2][256];
+    __shared__ unsigned pairs;
+    red[0][threadIdx.x] = moving.value() + rest_ke * rest.k.value();
+    red[1][threadIdx.x] = q * charge.k.value();
+    if (threadIdx.x == 0) pairs = 0;
     __syncthreads();
+    npair = __reduce_add_sync(0xffffffffu, npair);
+    if ((threadIdx.x & 31u) == 0u) atomicAdd(&pairs, npair);
     for (int off = blockDim.x / 2; off > 0; off >>= 1) {
         if ((int)threadIdx.x < off) {
             red[0][threadIdx.x] += red[0][threadIdx.x + off];
             red[1][threadIdx.x] += red[1][threadIdx.x + off];
-            red[2][threadIdx.x] += red[2][threadIdx.x + off];
         }
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        partials[3 * blockIdx.x] = red[0][0];
-        partials[3 * blockIdx.x + 1] = red[1][0];
-        partials[3 * blockIdx.x + 2] = red[2][0];
+        partials[4 * blockIdx.x] = red[0][0];
+        partials[4 * blockIdx.x + 1] = red[1][0];
+        partials[4 * blockIdx.x + 2] = (double)pairs;
+        partials[4 * blockIdx.x + 3] = overflow ? -1.0 : records;
     }
 }
 
+// returns the blocks whose partials (4 each) it writes: four per SM at most
+// (an idle block costs FP64 additions too)
 template <typename real>
-void launch_particle_sums(const Geom &g, const Species<real> &sp, const int *lo, const int *hi, double q,
-                          const real u_drift[3], double *partials, int nblocks, cudaStream_t s)
+int launch_particle_sums(const Geom &g, const Species<real> &sp, const int *lo, const int *hi, double q, real u_drift,
+                         double *partials, int max_blocks, cudaStream_t s)
 {
-    particle_sums_kernel<real><<<nblocks, 256, 0, s>>>(g, sp, lo, hi, q, (double)u_drift[0], (double)u_drift[1],
-                                                       (double)u_drift[2], partials);
+    const int64_t cap = std::min<int64_t>(max_blocks, (int64_t)device_sms() * 4);
+    const int nblocks = (int)std::min(cap, g.ntiles);
+    const double u = (double)u_drift;
+    particle_sums_kernel<real><<<nblocks, 256, 0, s>>>(g, sp, lo, hi, q, u, u * u / (std::sqrt(1.0 + u * u) + 1.0),
+                                                       partials);
+    return nblocks;
 }
 
 #define PIC_INSTANTIATE(real)                                                                       \
@@ -439,8 +467,8 @@ void launch_particle_sums(const Geom &g, const Species<real> &sp, const int *lo,
     template void launch_sort_cells<real>(const SortArgs<real> &, cudaStream_t);                    \
     template void launch_rho<real>(const Geom &, const Species<real> &, const int *, const int *, real, \
                                    real *, cudaStream_t);                                            \
-    template void launch_particle_sums<real>(const Geom &, const Species<real> &, const int *,      \
-                                             const int *, double, const real *, double *, int,      \
+    template int launch_particle_sums<real>(const Geom &, const Species<real> &, const int *,      \
+                                             const int *, double, real, double *, int,      \
                                              cudaStream_t);
 PIC_INSTANTIATE(float)
 PIC_INSTANTIATE(double)
