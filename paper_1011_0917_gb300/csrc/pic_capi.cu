@@ -216,15 +216,14 @@ static void side_raw(pic_ctx *c, int sp, int sidx, bool flat, void *out[kAttrs])
         out[a] = L.off[a] == SIZE_MAX ? nullptr : (void *)(base + (flat ? L.off[a] : L.boff[a]));
 }
 
+// a view of attribute pointers: sr, sc as in Species (32: flat arrays)
 template <typename real>
-static Species<real> species_view(pic_ctx *c, int sp, int sidx, bool flat = false)
+static Species<real> view_of(void *const p[kAttrs], int sr, int sc)
 {
     Species<real> s{};
-    void *p[kAttrs];
-    side_raw(c, sp, sidx, flat, p);
     auto at = [&](int a) -> void * { return p[a]; };
-    s.sr = flat ? 32 : (int)(c->side[sp].rb / sizeof(real));
-    s.sc = flat ? 32 : (int)(c->side[sp].rb / 4);
+    s.sr = sr;
+    s.sc = sc;
     s.ox = (real *)at(0);
     s.oy = (real *)at(1);
     s.oz = (real *)at(2);
@@ -238,6 +237,14 @@ static Species<real> species_view(pic_ctx *c, int sp, int sidx, bool flat = fals
     s.dly = (real *)at(10);
     s.dlz = (real *)at(11);
     return s;
+}
+
+template <typename real>
+static Species<real> species_view(pic_ctx *c, int sp, int sidx, bool flat = false)
+{
+    void *p[kAttrs];
+    side_raw(c, sp, sidx, flat, p);
+    return view_of<real>(p, flat ? 32 : (int)(c->side[sp].rb / sizeof(real)), flat ? 32 : (int)(c->side[sp].rb / 4));
 }
 
 static cudaMemcpyKind kind_out(int dst_is_device) { return dst_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost; }
@@ -617,14 +624,13 @@ static bool host_to_cell(double x, double h, int n, bool periodic, int &cell, re
     return true;
 }
 
-// bucket slots [0, n) of the inactive (staging) side into the active side
+// bucket n records of a flat list on the device into the active side
 template <typename real>
-static pic_status bucket_staged(pic_ctx *c, int sp, int64_t n)
+static pic_status bucket_flat(pic_ctx *c, int sp, int64_t n, const Species<real> &src)
 {
-    const int stage = c->cur[sp] ^ 1;
     BucketArgs<real> b{};
     b.g = c->g;
-    b.src = species_view<real>(c, sp, stage, true);
+    b.src = src;
     b.dst = species_view<real>(c, sp, c->cur[sp]);
     b.n = n;
     b.dst_hi = counts(c, sp, c->cur[sp], 1);
@@ -634,10 +640,19 @@ static pic_status bucket_staged(pic_ctx *c, int sp, int64_t n)
     return check_device_error(c);
 }
 
-// copy flat columns (host or device) into the staging side, then bucket them
+// bucket flat columns: from where they are when the device can read them
+// there, else through a copy in the staging (inactive) side
 template <typename real>
 static pic_status upload_flat(pic_ctx *c, int sp, int64_t n, const void *const cols[kAttrs], int src_is_device)
 {
+    bool direct = src_is_device != 0;
+    void *own[kAttrs] = {nullptr};
+    for (int a = 0; a < kAttrs; ++a) {
+        if (c->side[sp].off[a] == SIZE_MAX) continue;
+        own[a] = const_cast<void *>(cols[a]);
+        direct = direct && cols[a] && (uintptr_t)cols[a] % attr_size(c, a) == 0;
+    }
+    if (direct) return bucket_flat<real>(c, sp, n, view_of<real>(own, 32, 32));
     void *dst[kAttrs];
     side_raw(c, sp, c->cur[sp] ^ 1, true, dst);
     for (int a = 0; a < kAttrs; ++a) {
@@ -646,7 +661,7 @@ static pic_status upload_flat(pic_ctx *c, int sp, int64_t n, const void *const c
         if (bytes == 0) continue;
         CUDA_TRY(c, cudaMemcpyAsync(dst[a], cols[a], bytes, kind_in(src_is_device), c->stream));
     }
-    return bucket_staged<real>(c, sp, n);
+    return bucket_flat<real>(c, sp, n, species_view<real>(c, sp, c->cur[sp] ^ 1, true));
 }
 
 template <typename real>
