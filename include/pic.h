@@ -624,11 +624,10 @@ pic_status pic_filter_current_noalloc(int dim, int nx, int ny, int nz, int bc_z,
 
 /* ------------------------------------------------------- bounded waits */
 
-/* Kernels that stage data with the tensor memory accelerator wait on
-   mbarriers; no such wait spins without limit: it gives up after a time
-   budget, the kernel stops issuing work, and the step reports
-   PIC_ERR_TIMEOUT instead of hanging.  This call checks that path on the
-   device: one CTA waits on an mbarrier that expects one arrival, which the
+/* The library's wait on an mbarrier never spins without limit: it gives up
+   after a time budget, and its caller reports PIC_ERR_TIMEOUT instead of
+   hanging (no kernel of the step waits on one at present).  This call checks
+   the wait on the device: one CTA waits on an mbarrier that expects one arrival, which the
    kernel makes (arrive = 1: PIC_OK) or withholds (arrive = 0: nothing ever
    completes the phase, the wait runs out after budget_ms and the call
    returns PIC_ERR_TIMEOUT).  No fault is raised either way.  budget_ms in

@@ -1063,13 +1063,12 @@ static void run_phases_t(pic_ctx *c, unsigned mask)
     if ((mask & PIC_PH_FILTER) && c->p.filter_passes > 0) {
         PhaseTimer pt(c, 4);
         real *J[3] = {F[6], F[7], F[8]};
-        unsigned *err = reinterpret_cast<unsigned *>(c->scratch + c->off_err);
         if (!raw_in_tmp) {
-            launch_filter<real>(c->g, J, tmp, c->p.filter_passes, c->stream, err);
-        } else if (!launch_filter_from<real>(c->g, tmp, J, c->p.filter_passes, c->stream, err) &&
+            launch_filter<real>(c->g, J, tmp, c->p.filter_passes, c->stream);
+        } else if (!launch_filter_from<real>(c->g, tmp, J, c->p.filter_passes, c->stream) &&
                    !record_unsupported()) {
             cudaMemcpyAsync(J[0], tmp, (size_t)3 * c->g.ncomp * sizeof(real), cudaMemcpyDeviceToDevice, c->stream);
-            launch_filter<real>(c->g, J, tmp, c->p.filter_passes, c->stream, err);
+            launch_filter<real>(c->g, J, tmp, c->p.filter_passes, c->stream);
         }
         c->kernels += c->p.filter_passes <= 4 ? 1 : (int64_t)(c->g.dim == 3 ? 3 : 2) * c->p.filter_passes;
     }

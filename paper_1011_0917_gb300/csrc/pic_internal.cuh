@@ -780,12 +780,11 @@ void launch_yee(const Geom &g, real *const F[9], real *const F1[6], double dt, d
                 cudaStream_t s);
 // (err: the device error word for a bounded wait that ran out; may be null)
 template <typename real>
-void launch_filter(const Geom &g, real *const J[3], real *tmp, int npass, cudaStream_t s, unsigned *err = nullptr);
+void launch_filter(const Geom &g, real *const J[3], real *tmp, int npass, cudaStream_t s);
 // all passes from src (3 contiguous components, left unchanged) into J;
 // false (nothing launched) where only the per-pass path applies (npass > 4)
 template <typename real>
-bool launch_filter_from(const Geom &g, const real *src, real *const J[3], int npass, cudaStream_t s,
-                        unsigned *err = nullptr);
+bool launch_filter_from(const Geom &g, const real *src, real *const J[3], int npass, cudaStream_t s);
 // j0p non-null: the amplitude is read from device memory (a captured step)
 template <typename real>
 void launch_antenna(const Geom &g, real *J, int pol, int ka, double j0, double hx, double hy,
