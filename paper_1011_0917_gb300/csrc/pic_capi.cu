@@ -1718,17 +1718,30 @@ static pic_status get_fields_lab_t(pic_ctx *c, unsigned mask, unsigned char *dst
     const size_t per = (size_t)c->g.ncomp * c->es;
     real *tmp = reinterpret_cast<real *>(c->scratch + c->off_tmp);
     static const int partner[6] = {4, 3, -1, 1, 0, -1};  // By, Bx, -, Ey, Ex, -
+    LabArgs<real> a{};
+    a.g = c->g;
+    a.gam = c->gam;
+    a.beta = c->beta;
+    // to the device in one launch, to the host through one component of scratch
+    int n = 0;
     size_t o = 0;
     for (int q = 0; q < 6; ++q) {
         if (!(mask >> q & 1u)) continue;
-        real *out = dst_is_device ? reinterpret_cast<real *>(dst + o) : tmp;
-        const real *F = (const real *)field_ptr(c, q);
-        const real *P = partner[q] >= 0 ? (const real *)field_ptr(c, partner[q]) : F;
-        launch_lab_fields<real>(c->g, F, P, q, out, c->gam, c->beta, c->sms, c->stream);
-        CUDA_TRY(c, cudaGetLastError());
-        if (!dst_is_device) CUDA_TRY(c, cudaMemcpyAsync(dst + o, tmp, per, cudaMemcpyDeviceToHost, c->stream));
+        a.comp[n] = q;
+        a.F[n] = (const real *)field_ptr(c, q);
+        a.P[n] = partner[q] >= 0 ? (const real *)field_ptr(c, partner[q]) : a.F[n];
+        a.out[n] = dst_is_device ? reinterpret_cast<real *>(dst + o) : tmp;
+        if (dst_is_device) {
+            ++n;
+        } else {
+            launch_lab_fields<real>(a, 1, c->sms, c->stream);
+            CUDA_TRY(c, cudaGetLastError());
+            CUDA_TRY(c, cudaMemcpyAsync(dst + o, tmp, per, cudaMemcpyDeviceToHost, c->stream));
+        }
         o += per;
     }
+    if (n > 0) launch_lab_fields<real>(a, n, c->sms, c->stream);
+    CUDA_TRY(c, cudaGetLastError());
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
     return PIC_OK;
 }

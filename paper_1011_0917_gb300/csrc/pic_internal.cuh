@@ -401,6 +401,61 @@ __device__ __forceinline__ real drift_velocity(const Drift<real> &d, real dux, r
     return (duz * (real(2) + E) - d.U * p2) * (ig * d.ig * is);
 }
 
+// An unevaluated sum h + l of two FP32 values, |l| <= ulp(h) / 2: about 48
+// bits, from the error-free sum and product (Knuth, TAOCP 2, 4.2.2; Dekker,
+// Numer. Math. 18, 1971, with a fused multiply-add for the product's error).
+// FP64 arithmetic gives 2 lanes per SM and cycle here, FP32 128, of which one
+// of these operations takes 7 to 11.  The currents of records in relative
+// form use them: they need the records' exact positions and far more than
+// FP32's bits (see rel_actual), and end in fixed-point words that carry at
+// most 43.
+struct ff {
+    float h, l;
+    __device__ __forceinline__ ff() {}
+    __device__ __forceinline__ ff(float x) : h(x), l(0.0f) {}
+    __device__ __forceinline__ ff(int x) : h((float)x), l(0.0f) {}
+    __device__ __forceinline__ ff(double x) : h((float)x), l((float)(x - (double)(float)x)) {}
+    __device__ __forceinline__ ff(float x, float y) : h(x), l(y) {}
+};
+__device__ __forceinline__ ff two_sum(float a, float b)
+{
+    const float s = __fadd_rn(a, b), z = __fsub_rn(s, a);
+    return ff(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z)));
+}
+// |a| >= |b| or a = 0
+__device__ __forceinline__ ff quick_sum(float a, float b)
+{
+    const float s = __fadd_rn(a, b);
+    return ff(s, __fsub_rn(b, __fsub_rn(s, a)));
+}
+__device__ __forceinline__ ff operator+(ff a, ff b)
+{
+    const ff s = two_sum(a.h, b.h);
+    return quick_sum(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ ff operator-(ff a) { return ff(-a.h, -a.l); }
+__device__ __forceinline__ ff operator-(ff a, ff b) { return a + -b; }
+__device__ __forceinline__ ff operator*(ff a, ff b)
+{
+    const float p = __fmul_rn(a.h, b.h);
+    float e = __fmaf_rn(a.h, b.h, -p);
+    e = __fmaf_rn(a.h, b.l, e);
+    e = __fmaf_rn(a.l, b.h, e);
+    return quick_sum(p, e);
+}
+__device__ __forceinline__ ff &operator+=(ff &a, ff b)
+{
+    a = a + b;
+    return a;
+}
+__device__ __forceinline__ bool operator==(ff a, ff b) { return a.h == b.h && a.l == b.l; }
+// the exact floor (the low word decides where the high one is an integer)
+__device__ __forceinline__ float floor_ff(ff a)
+{
+    const float f = floorf(a.h);
+    return a.h == f && a.l < 0.0f ? f - 1.0f : f;
+}
+
 // Sums of many values of the working precision in FP64, compensated.  The
 // FP64 pipe takes 2 lanes per SM and cycle, so an FP32 value is not converted
 // and added by itself: up to kSumRun of them go into an unevaluated sum of
@@ -760,11 +815,17 @@ int launch_particle_sums(const Geom &g, const Species<real> &sp, const int *lo, 
 void launch_inject(const InjectArgs &a, cudaStream_t s);
 template <typename real>
 void launch_btd(const BtdArgs<real> &a, cudaStream_t s);
-// component comp (0..5) of the lab-frame E, B on the grid (F the component,
-// P its partner: By, Bx, -, Ey, Ex, -) into out; FP64 transformation
+// n components of the lab-frame E, B on the grid (comp[q] in 0..5, F the
+// component, P its partner: By, Bx, -, Ey, Ex, -) into out[q]
 template <typename real>
-void launch_lab_fields(const Geom &g, const real *F, const real *P, int comp, real *out, double gam, double beta,
-                       int sms, cudaStream_t s);
+struct LabArgs {
+    Geom g;
+    int comp[6];
+    const real *F[6], *P[6];
+    real *out[6];
+    double gam, beta;
+};
+template <typename real> void launch_lab_fields(const LabArgs<real> &a, int n, int sms, cudaStream_t s);
 // moving window: every field plane k of dst takes plane k + S of src (zero
 // above), for the nine components
 template <typename real>

@@ -121,60 +121,6 @@ __device__ __forceinline__ void sh_acc2(int *p, f32x2 a, f32x2 b, f32x2 lo_scale
     sh_add(p + LOFF + STRIDE, (int)(unsigned)(l >> 32) - kRoundMagicBits);
 }
 
-// An unevaluated sum h + l of two FP32 values, |l| <= ulp(h) / 2: about 48
-// bits, from the error-free sum and product (Knuth, TAOCP 2, 4.2.2; Dekker,
-// Numer. Math. 18, 1971, with a fused multiply-add for the product's error).
-// The currents of records in relative form need their exact positions and far
-// more than FP32's bits (see rel_actual), and end in fixed-point words that
-// carry at most 43 bits; FP64 arithmetic gives 2 lanes per SM and cycle here,
-// FP32 128, of which one of these operations takes 7 to 11.
-struct ff {
-    float h, l;
-    __device__ __forceinline__ ff() {}
-    __device__ __forceinline__ ff(float x) : h(x), l(0.0f) {}
-    __device__ __forceinline__ ff(int x) : h((float)x), l(0.0f) {}
-    __device__ __forceinline__ ff(double x) : h((float)x), l((float)(x - (double)(float)x)) {}
-    __device__ __forceinline__ ff(float x, float y) : h(x), l(y) {}
-};
-__device__ __forceinline__ ff two_sum(float a, float b)
-{
-    const float s = __fadd_rn(a, b), z = __fsub_rn(s, a);
-    return ff(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z)));
-}
-// |a| >= |b| or a = 0
-__device__ __forceinline__ ff quick_sum(float a, float b)
-{
-    const float s = __fadd_rn(a, b);
-    return ff(s, __fsub_rn(b, __fsub_rn(s, a)));
-}
-__device__ __forceinline__ ff operator+(ff a, ff b)
-{
-    const ff s = two_sum(a.h, b.h);
-    return quick_sum(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
-}
-__device__ __forceinline__ ff operator-(ff a) { return ff(-a.h, -a.l); }
-__device__ __forceinline__ ff operator-(ff a, ff b) { return a + -b; }
-__device__ __forceinline__ ff operator*(ff a, ff b)
-{
-    const float p = __fmul_rn(a.h, b.h);
-    float e = __fmaf_rn(a.h, b.h, -p);
-    e = __fmaf_rn(a.h, b.l, e);
-    e = __fmaf_rn(a.l, b.h, e);
-    return quick_sum(p, e);
-}
-__device__ __forceinline__ ff &operator+=(ff &a, ff b)
-{
-    a = a + b;
-    return a;
-}
-__device__ __forceinline__ bool operator==(ff a, ff b) { return a.h == b.h && a.l == b.l; }
-// the exact floor (the low word decides where the high one is an integer)
-__device__ __forceinline__ float floor_ff(ff a)
-{
-    const float f = floorf(a.h);
-    return a.h == f && a.l < 0.0f ? f - 1.0f : f;
-}
-
 // contributions of records in relative form into the same fixed-point words
 template <int LOFF>
 __device__ __forceinline__ void sh_acc(int *p, ff a, ff b, ff lo_scale)
