@@ -366,6 +366,7 @@ template <typename real, int DIM> struct AdjBlocks {
 template <typename real, int DIM, int S>
 __global__ void __launch_bounds__(256, (AdjBlocks<real, DIM>::push)) adj_push_kernel(AdjArgs<real> a)
 {
+    chain_begin();
     constexpr int W = S + 2, WY = DIM == 3 ? W : 1;
     const Geom &g = a.g;
     const Drift<real> drift(a.u_drift, a.dtdh[2]);
@@ -534,6 +535,7 @@ __device__ __forceinline__ real adj_ion_vjp_one(const AdjArgs<real> &a, const Dr
 template <typename real, int DIM, int S>
 __global__ void __launch_bounds__(256, (AdjBlocks<real, DIM>::vjp)) adj_push_vjp_kernel(AdjArgs<real> a)
 {
+    chain_begin();
     constexpr int W = S + 2, WY = DIM == 3 ? W : 1;
     const Geom &g = a.g;
     const Drift<real> drift(a.u_drift, a.dtdh[2]);
@@ -827,8 +829,12 @@ __global__ void __launch_bounds__(256, (AdjBlocks<real, DIM>::vjp)) adj_push_vjp
 // scatter of every B update onto the E nodes it read (hy_ unused in 2D).
 template <typename real>
 __global__ void adj_curl_e_t_kernel(Geom g, real *lEx, real *lEy, real *lEz, const real *lBx, const real *lBy,
-                                    const real *lBz, real hz_, real hx_, real hy_)
+                                    const real *lBz, real hz_, real hx_, real hy_, unsigned char *near, int nz1)
 {
+    chain_begin();
+    // (the masks the reverse step sets later start from zero)
+    if (near)
+        for (int k = (int)(blockIdx.x * blockDim.x + threadIdx.x); k < nz1; k += (int)(gridDim.x * blockDim.x)) near[k] = 0;
     const bool per = g.bc_z == 0, d3 = g.dim == 3;
     const int nk = per ? g.nz : g.nz + 1;
     const int64_t plane = g.plane;
@@ -864,6 +870,7 @@ __global__ void adj_e_update_t_kernel(Geom g, const real *lE1x, const real *lE1y
                                       real *pEy, real *pEz, real *lE0x, real *lE0y, real *lE0z, real *lJx,
                                       real *lJy, real *lJz, real cm, real m2pidt)
 {
+    chain_begin();
     const bool per = g.bc_z == 0;
     const int nk = g.nz + 1;
     const int64_t plane = g.plane;
@@ -906,6 +913,7 @@ template <typename real>
 __global__ void adj_curl_b_t_kernel(Geom g, const real *pEx, const real *pEy, const real *pEz, real *lBx,
                                     real *lBy, real *lBz, real dthz, real dthx, real dthy)
 {
+    chain_begin();
     const bool per = g.bc_z == 0, d3 = g.dim == 3;
     const int nk = g.nz + 1;
     const int64_t plane = g.plane;
@@ -939,6 +947,7 @@ template <typename real>
 __global__ void adj_antenna_kernel(Geom g, const real *lJ, int pol, int ka, double hx, double hy, double xc,
                                    double yc, double inv_w2, double fa, double fw, double *s)
 {
+    chain_begin();
     double s0 = 0, s1 = 0;
     for (int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; o < g.plane;
          o += (int64_t)gridDim.x * blockDim.x) {
@@ -1036,6 +1045,7 @@ __device__ __forceinline__ bool any_nonzero(const real *P, int n, int first, int
 template <typename real, bool WARP>
 __global__ void adj_planes_kernel(Geom g, const real *F, int nc, unsigned char *near)
 {
+    chain_begin();
     const int nk = g.bc_z == 0 ? g.nz : g.nz + 1, n = nk * nc;
     const int per = WARP ? (int)(blockDim.x >> 5) : 1, mine = WARP ? (int)(threadIdx.x >> 5) : 0;
     const int first = WARP ? (int)(threadIdx.x & 31u) : (int)threadIdx.x, stride = WARP ? 32 : (int)blockDim.x;
@@ -1052,13 +1062,12 @@ __global__ void adj_planes_kernel(Geom g, const real *F, int nc, unsigned char *
 template <typename real>
 void launch_adj_planes(const Geom &g, const real *F, int nc, unsigned char *near, cudaStream_t s)
 {
-    cudaMemsetAsync(near, 0, (size_t)g.nz + 1, s);
     const int n = (g.nz + 1) * nc, cap = device_sms() * 32;
     if (g.plane <= kWarpPlane) {
         const int blocks = (n + 3) / 4;
-        adj_planes_kernel<real, true><<<(unsigned)(blocks < cap ? blocks : cap), 128, 0, s>>>(g, F, nc, near);
+        launch_chained(chained(g), adj_planes_kernel<real, true>, (unsigned)(blocks < cap ? blocks : cap), 128, 0, s, g, F, nc, near);
     } else {
-        adj_planes_kernel<real, false><<<(unsigned)(n < cap ? n : cap), 128, 0, s>>>(g, F, nc, near);
+        launch_chained(chained(g), adj_planes_kernel<real, false>, (unsigned)(n < cap ? n : cap), 128, 0, s, g, F, nc, near);
     }
 }
 
@@ -1068,11 +1077,11 @@ void launch_adj_planes(const Geom &g, const real *F, int nc, unsigned char *near
     if (a.n <= 0) return;                                                                       \
     const unsigned grid = adj_grid(a.n, 256);                                                   \
     if (a.g.dim == 3) {                                                                         \
-        if (a.g.shape == 1) kernel<real, 3, 1><<<grid, 256, 0, s>>>(a);                         \
-        else kernel<real, 3, 2><<<grid, 256, 0, s>>>(a);                                        \
+        if (a.g.shape == 1) launch_chained(chained(a.g), kernel<real, 3, 1>, grid, 256, 0, s, a);                         \
+        else launch_chained(chained(a.g), kernel<real, 3, 2>, grid, 256, 0, s, a);                                        \
     } else {                                                                                    \
-        if (a.g.shape == 1) kernel<real, 2, 1><<<grid, 256, 0, s>>>(a);                         \
-        else kernel<real, 2, 2><<<grid, 256, 0, s>>>(a);                                        \
+        if (a.g.shape == 1) launch_chained(chained(a.g), kernel<real, 2, 1>, grid, 256, 0, s, a);                         \
+        else launch_chained(chained(a.g), kernel<real, 2, 2>, grid, 256, 0, s, a);                                        \
     }
 
 template <typename real>
@@ -1093,29 +1102,29 @@ void launch_adj_push_vjp(const AdjArgs<real> &a, cudaStream_t s)
 // cotangent of the filtered current); lE0 and pE are work components
 template <typename real>
 void launch_adj_yee(const Geom &g, real *lE[3], real *lB[3], real *lE0[3], real *pE[3], real *lJ[3], double dt,
-                    double hx, double hy, double hz, cudaStream_t s)
+                    double hx, double hy, double hz, unsigned char *near, cudaStream_t s)
 {
     const unsigned grid = adj_grid((int64_t)(g.nz + 1) * g.plane, 256);
     const real h = (real)(0.5 * dt);
     // B^{n+1} = B' - h curl E^{n+1}
-    adj_curl_e_t_kernel<real><<<grid, 256, 0, s>>>(g, lE[0], lE[1], lE[2], lB[0], lB[1], lB[2], (real)(h / hz),
-                                                  (real)(h / hx), (real)(h / hy));
+    launch_chained(chained(g), adj_curl_e_t_kernel<real>, grid, 256, 0, s, g, lE[0], lE[1], lE[2], lB[0], lB[1], lB[2], (real)(h / hz),
+                                                  (real)(h / hx), (real)(h / hy), near, g.nz + 1);
     // E^{n+1} = E^n + dt (curl B' - 2 pi J), Mur on the z ends
-    adj_e_update_t_kernel<real><<<grid, 256, 0, s>>>(g, lE[0], lE[1], lE[2], pE[0], pE[1], pE[2], lE0[0], lE0[1],
+    launch_chained(chained(g), adj_e_update_t_kernel<real>, grid, 256, 0, s, g, lE[0], lE[1], lE[2], pE[0], pE[1], pE[2], lE0[0], lE0[1],
                                                     lE0[2], lJ[0], lJ[1], lJ[2], (real)((dt - hz) / (dt + hz)),
                                                     (real)(-kTwoPiD * dt));
-    adj_curl_b_t_kernel<real><<<grid, 256, 0, s>>>(g, pE[0], pE[1], pE[2], lB[0], lB[1], lB[2], (real)(dt / hz),
+    launch_chained(chained(g), adj_curl_b_t_kernel<real>, grid, 256, 0, s, g, pE[0], pE[1], pE[2], lB[0], lB[1], lB[2], (real)(dt / hz),
                                                   (real)(dt / hx), (real)(dt / hy));
     // B' = B^n - h curl E^n
-    adj_curl_e_t_kernel<real><<<grid, 256, 0, s>>>(g, lE0[0], lE0[1], lE0[2], lB[0], lB[1], lB[2], (real)(h / hz),
-                                                  (real)(h / hx), (real)(h / hy));
+    launch_chained(chained(g), adj_curl_e_t_kernel<real>, grid, 256, 0, s, g, lE0[0], lE0[1], lE0[2], lB[0], lB[1], lB[2], (real)(h / hz),
+                                                  (real)(h / hx), (real)(h / hy), (unsigned char *)nullptr, 0);
 }
 
 template <typename real>
 void launch_adj_antenna(const Geom &g, const real *lJ, int pol, int ka, double hx, double hy, double xc, double yc,
                         double waist, double fa, double fw, double *s, cudaStream_t st)
 {
-    adj_antenna_kernel<real><<<adj_grid(g.plane, 256), 256, 0, st>>>(g, lJ, pol, ka, hx, hy, xc, yc,
+    launch_chained(chained(g), adj_antenna_kernel<real>, adj_grid(g.plane, 256), 256, 0, st, g, lJ, pol, ka, hx, hy, xc, yc,
                                                                       1.0 / (waist * waist), fa, fw, s);
 }
 
@@ -1129,7 +1138,7 @@ void launch_adj_profile(int64_t n, const double *lw, const void *w, int precisio
     template void launch_adj_push<real>(const AdjArgs<real> &, cudaStream_t);                                  \
     template void launch_adj_push_vjp<real>(const AdjArgs<real> &, cudaStream_t);                              \
     template void launch_adj_yee<real>(const Geom &, real *[3], real *[3], real *[3], real *[3], real *[3],     \
-                                       double, double, double, double, cudaStream_t);                          \
+                                       double, double, double, double, unsigned char *, cudaStream_t);                          \
     template void launch_adj_planes<real>(const Geom &, const real *, int, unsigned char *, cudaStream_t);     \
     template void launch_adj_antenna<real>(const Geom &, const real *, int, int, double, double, double, double, \
                                            double, double, double, double *, cudaStream_t);

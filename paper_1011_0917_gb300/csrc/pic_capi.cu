@@ -21,6 +21,7 @@ using namespace pic;
 
 namespace pic {
 thread_local BatchRecorder *g_rec = nullptr;
+thread_local bool g_capture = false;
 
 int device_sms()
 {
@@ -1011,6 +1012,7 @@ static void run_phases_t(pic_ctx *c, unsigned mask)
     if (mask & PIC_PH_ZERO_J) {
         PhaseTimer pt(c, 0);
         launch_zero<real>(R[0], (int64_t)3 * c->g.ncomp, c->stream);
+        c->kernels += 1;
     }
     // With ions paired to their electrons, the electron kernel also takes the
     // tile's drifting ion records, so electron and ion currents add in one
@@ -1413,6 +1415,7 @@ static pic_status batch_capture(pic_batch *b, int K)
         if (st != PIC_OK || ok) return st;
     }
     if (bad(cudaStreamBeginCapture(G.cs, cudaStreamCaptureModeRelaxed))) return PIC_ERR_CUDA;
+    g_capture = true;
     cudaEventRecord(G.join, G.cs);
     for (size_t i = 0; i < nctx; ++i) cudaStreamWaitEvent(b->ctx[i]->stream, G.join, 0);
     std::vector<int64_t> k0(nctx);
@@ -1431,6 +1434,7 @@ static pic_status batch_capture(pic_batch *b, int K)
         cudaEventRecord(G.ev[i], b->ctx[i]->stream);
         cudaStreamWaitEvent(G.cs, G.ev[i], 0);
     }
+    g_capture = false;
     const cudaError_t e = cudaStreamEndCapture(G.cs, &G.graph);
     // the capture flipped every double buffer K times (K even: back where it
     // was) and counted the kernels of K steps, which every replay adds
@@ -2447,7 +2451,7 @@ static void adj_step(pic_ctx *c, const AdjLayout &L, unsigned char *sa, unsigned
     const int64_t nc = c->g.ncomp;
     // the raw current goes to the filter's input buffer; the filter writes J
     real *J = (real *)(B + L.J), *R = (real *)(B + L.tmp);
-    cudaMemsetAsync(R, 0, 3 * sizeof(real) * nc, c->stream);
+    launch_zero2<real>(R, 3 * nc, sa + L.fm, c->g.nz + 1, c->stream);
     AdjArgs<real> a{};
     a.g = c->g;
     for (int q = 0; q < 3; ++q) {
@@ -2627,7 +2631,7 @@ static pic_status adj_backward_t(pic_ctx *c, const void *cot)
             const int n = n0 + s;
             // the current cotangent before the filter goes to the scratch
             // buffer, the filter (its own transpose) writes lJ
-            launch_adj_yee<real>(c->g, lE, lB, lE0, pE, lJr, c->dt, c->hx, c->hy, c->hz, c->stream);
+            launch_adj_yee<real>(c->g, lE, lB, lE0, pE, lJr, c->dt, c->hx, c->hy, c->hz, B + L.planes, c->stream);
             for (int q = 0; q < 3; ++q) std::swap(lE[q], lE0[q]);
             if (c->p.filter_passes == 0 || !launch_filter_from<real>(c->g, lJr[0], lJ, c->p.filter_passes, c->stream)) {
                 CUDA_TRY(c, cudaMemcpyAsync(lJ[0], lJr[0], 3 * sizeof(real) * nc, cudaMemcpyDeviceToDevice, c->stream));

@@ -633,6 +633,7 @@ __device__ __forceinline__ void yee3d_item(const YeeArgs<real> &a, int64_t item)
 template <typename real>
 __global__ void __launch_bounds__(512, 2) yee3d_kernel(YeeArgs<real> a)
 {
+    chain_begin();
     yee3d_item(a, (int64_t)blockIdx.x);
 }
 
@@ -666,6 +667,7 @@ __device__ __forceinline__ void yee2d_items(const YeeArgs<real> &a, int64_t item
 template <typename real>
 __global__ void __launch_bounds__(256) yee2d_kernel(YeeArgs<real> a, int64_t nitems)
 {
+    chain_begin();
     yee2d_items(a, (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5), nitems);
 }
 
@@ -717,7 +719,7 @@ void launch_yee(const Geom &g, real *const F[9], real *const F1[6], double dt, d
         a.nchunks = (nzo + a.cz - 1) / a.cz;
         const int64_t nitems = (int64_t)nstrip * a.nchunks, nblocks = (nitems + 7) / 8;
         if (record_launch(kBPYee, launch_yee2d_batch<real>, a, nblocks)) return;
-        yee2d_kernel<real><<<(unsigned)nblocks, 256, 0, s>>>(a, nitems);
+        launch_chained(chained(g), yee2d_kernel<real>, (unsigned)nblocks, 256, 0, s, a, nitems);
         return;
     }
     {
@@ -726,7 +728,7 @@ void launch_yee(const Geom &g, real *const F[9], real *const F1[6], double dt, d
         a.nchunks = (nzo + a.cz - 1) / a.cz;
         const int64_t nblocks = ncol * a.nchunks;
         if (record_launch(kBPYee, launch_yee3d_batch<real>, a, nblocks)) return;
-        yee3d_kernel<real><<<(unsigned)nblocks, 512, 0, s>>>(a);
+        launch_chained(chained(g), yee3d_kernel<real>, (unsigned)nblocks, 512, 0, s, a);
     }
 }
 
@@ -1082,6 +1084,7 @@ template <typename real, int H>
 __global__ void __launch_bounds__(512, (sizeof(real) == 4 && H <= 2 ? 2 : 1))
     filter3d_kernel(Geom g, const real *in, real *out, int cz, int nchunks)
 {
+    chain_begin();
     filter3d_item<real, H>(g, in, out, cz, nchunks, (int64_t)blockIdx.x);
 }
 
@@ -1115,6 +1118,7 @@ __device__ __forceinline__ void filter2d_items(const Geom &g, const real *in, re
 template <typename real, int H>
 __global__ void __launch_bounds__(256) filter2d_kernel(Geom g, const real *in, real *out, int cz, int nchunks)
 {
+    chain_begin();
     filter2d_items<real, H>(g, in, out, cz, nchunks, (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5));
 }
 
@@ -1152,7 +1156,7 @@ static void launch_march(const Geom &g, const real *in, real *out, cudaStream_t 
         if (record_launch(kBPFilter, launch_filter2d_batch<real, H>, MarchArgs<real>{g, in, out, cz, nchunks},
                           nblocks))
             return;
-        filter2d_kernel<real, H><<<(unsigned)nblocks, 256, 0, s>>>(g, in, out, cz, nchunks);
+        launch_chained(chained(g), filter2d_kernel<real, H>, (unsigned)nblocks, 256, 0, s, g, in, out, cz, nchunks);
     } else {
         constexpr int OWN = 32 - 2 * H;
         const int64_t ncol = (int64_t)((g.nx + OWN - 1) / OWN) * ((g.ny + OWN - 1) / OWN);
@@ -1163,7 +1167,7 @@ static void launch_march(const Geom &g, const real *in, real *out, cudaStream_t 
         if (record_launch(kBPFilter, launch_filter3d_batch<real, H>, MarchArgs<real>{g, in, out, cz, nchunks},
                           nblocks))
             return;
-        filter3d_kernel<real, H><<<(unsigned)nblocks, 512, 0, s>>>(g, in, out, cz, nchunks);
+        launch_chained(chained(g), filter3d_kernel<real, H>, (unsigned)nblocks, 512, 0, s, g, in, out, cz, nchunks);
     }
 }
 
@@ -1264,6 +1268,7 @@ __device__ __forceinline__ void antenna_body(const AntennaArgs<real> &a, int64_t
 template <typename real>
 __global__ void antenna_kernel(AntennaArgs<real> a)
 {
+    chain_begin();
     antenna_body(a, (int64_t)blockIdx.x, (int64_t)gridDim.x);
 }
 
@@ -1291,7 +1296,7 @@ void launch_antenna(const Geom &g, real *J, int pol, int ka, double j0, double h
     const AntennaArgs<real> a{g, J, pol, ka, j0, hx, hy, xc, yc, 1.0 / (waist * waist), j0p};
     const unsigned nb = grid_for(g.plane, 256);
     if (record_launch(kBPAntenna, launch_antenna_batch<real>, a, (int64_t)nb)) return;
-    antenna_kernel<real><<<nb, 256, 0, s>>>(a);
+    launch_chained(chained(g), antenna_kernel<real>, (unsigned)nb, 256, 0, s, a);
 }
 
 // ---------------------------------------------------------------- zeroing
@@ -1316,13 +1321,44 @@ static void launch_zero_batch(const void *args, const int64_t *start, int n, int
     zero_batch_kernel<real><<<(unsigned)total, 256, 0, s>>>(static_cast<const ZeroArgs<real> *>(args), start, n);
 }
 
+// n values at p (16-byte aligned) and m bytes at q
+template <typename real>
+__global__ void __launch_bounds__(256) zero_kernel(real *p, int64_t n, unsigned char *q, int64_t m)
+{
+    chain_begin();
+    const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+    constexpr int V = 16 / (int)sizeof(real);
+    for (int64_t o = first; o < n / V; o += stride) reinterpret_cast<int4 *>(p)[o] = make_int4(0, 0, 0, 0);
+    for (int64_t o = n / V * V + first; o < n; o += stride) p[o] = real(0);
+    for (int64_t o = first; o < m; o += stride) q[o] = 0;
+}
+
+template <typename real>
+static void zero_launch(real *p, int64_t n, unsigned char *q, int64_t m, cudaStream_t s)
+{
+    // a large array, or one off the 16-byte grid (J of an odd grid, zeroed
+    // by itself): a plain memset
+    if (n > 3 * kChainNodes || reinterpret_cast<uintptr_t>(p) % 16 != 0) {
+        cudaMemsetAsync(p, 0, (size_t)n * sizeof(real), s);
+        n = 0;
+        if (m == 0) return;
+    }
+    launch_chained(true, zero_kernel<real>, grid_for(n / 4 + 1, 256), 256, 0, s, p, n, q, m);
+}
+
 template <typename real>
 void launch_zero(real *p, int64_t n, cudaStream_t s)
 {
     if (n <= 0) return;
     if (record_launch(kBPZero, launch_zero_batch<real>, ZeroArgs<real>{p, n}, (n + kZeroChunk - 1) / kZeroChunk))
         return;
-    cudaMemsetAsync(p, 0, (size_t)n * sizeof(real), s);
+    zero_launch(p, n, nullptr, 0, s);
+}
+
+template <typename real>
+void launch_zero2(real *p, int64_t n, unsigned char *q, int64_t m, cudaStream_t s)
+{
+    zero_launch(p, n, q, m, s);
 }
 
 // ------------------------------------------------------------ field sums
@@ -1392,7 +1428,8 @@ int launch_field_sums(const Geom &g, real *const F[9], double *partials, int max
     template void launch_antenna<real>(const Geom &, real *, int, int, double, double, double, double,  \
                                        double, double, cudaStream_t, const double *);                   \
     template int launch_field_sums<real>(const Geom &, real *const[9], double *, int, cudaStream_t); \
-    template void launch_zero<real>(real *, int64_t, cudaStream_t);
+    template void launch_zero<real>(real *, int64_t, cudaStream_t);                                     \
+    template void launch_zero2<real>(real *, int64_t, unsigned char *, int64_t, cudaStream_t);
 PIC_FIELDS_INSTANTIATE(float)
 PIC_FIELDS_INSTANTIATE(double)
 

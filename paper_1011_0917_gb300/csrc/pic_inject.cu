@@ -225,6 +225,7 @@ __device__ __forceinline__ void inject_body(const InjectArgs &a, const int64_t b
 template <typename real>
 __global__ void inject_kernel(InjectArgs a)
 {
+    chain_begin();
     inject_body<real>(a, (int64_t)blockIdx.x, (int64_t)gridDim.x);
 }
 
@@ -258,8 +259,8 @@ void launch_inject(const InjectArgs &a, cudaStream_t s)
     if (record_launch(kBPInject, a.precision == 0 ? launch_inject_batch<float> : launch_inject_batch<double>, a,
                       blocks))
         return;
-    if (a.precision == 0) inject_kernel<float><<<(unsigned)blocks, kInjectThreads, 0, s>>>(a);
-    else inject_kernel<double><<<(unsigned)blocks, kInjectThreads, 0, s>>>(a);
+    launch_chained(chained(a.g), a.precision == 0 ? inject_kernel<float> : inject_kernel<double>, (unsigned)blocks,
+                   kInjectThreads, 0, s, a);
 }
 
 }  // namespace pic

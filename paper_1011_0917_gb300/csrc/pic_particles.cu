@@ -13,6 +13,7 @@ template <typename real, int DIM, int S, int TX, int TY, int TZ, bool REL>
 __global__ void __launch_bounds__((BlockOf<real, DIM>::value), (MinBlocks<real, DIM>::value)) push_kernel(PushArgs<real> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    chain_begin();
     for (int64_t t = blockIdx.x; t < a.g.ntiles; t += gridDim.x) push_tile<real, DIM, S, TX, TY, TZ, REL>(a, t, smem_raw);
 }
 
@@ -22,6 +23,7 @@ template <typename real, int DIM, int S, int TX, int TY, int TZ, bool REL>
 __global__ void __launch_bounds__((BlockOf<real, DIM>::value)) ion_kernel(PushArgs<real> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    chain_begin();
     for (int64_t t = blockIdx.x; t < a.g.ntiles; t += gridDim.x) ion_tile<real, DIM, S, TX, TY, TZ, REL>(a, t, smem_raw);
 }
 
@@ -35,7 +37,7 @@ static void launch_push_z(const PushArgs<real> &a, bool ions, cudaStream_t s)
     auto k = ions ? ion_kernel<real, DIM, S, TX, TY, TZ, REL> : push_kernel<real, DIM, S, TX, TY, TZ, REL>;
     if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const int64_t grid = a.g.ntiles < 2147483647LL ? a.g.ntiles : 2147483647LL;
-    k<<<(unsigned)grid, BlockOf<real, DIM>::value, smem, s>>>(a);
+    launch_chained(chained(a.g), k, (unsigned)grid, BlockOf<real, DIM>::value, smem, s, a);
 }
 
 // records in relative form (and their ions) take the REL kernels
