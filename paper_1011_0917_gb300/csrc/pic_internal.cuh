@@ -775,21 +775,35 @@ __device__ __forceinline__ void chain_begin()
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+// (cluster: CTAs per thread-block cluster)
 template <typename... P, typename... A>
-inline void launch_chained(bool chain, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
-                           A... args)
+inline void launch_clusters(bool chain, unsigned cluster, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem,
+                            cudaStream_t s, A... args)
 {
     cudaLaunchConfig_t c{};
     c.gridDim = dim3(grid);
     c.blockDim = dim3(block);
     c.dynamicSmemBytes = smem;
     c.stream = s;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    c.attrs = &at;
-    c.numAttrs = chain && !g_capture ? 1 : 0;
+    cudaLaunchAttribute at[2] = {};
+    c.attrs = at;
+    if (chain && !g_capture) {
+        at[c.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[c.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        at[c.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        at[c.numAttrs].val.clusterDim.x = cluster;
+        at[c.numAttrs].val.clusterDim.y = 1;
+        at[c.numAttrs++].val.clusterDim.z = 1;
+    }
     (void)cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+template <typename... P, typename... A>
+inline void launch_chained(bool chain, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                           A... args)
+{
+    launch_clusters(chain, 1, kernel, grid, block, smem, s, args...);
 }
 
 // the run owning work item `item`: the last r with start[r] <= item

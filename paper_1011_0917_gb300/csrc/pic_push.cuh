@@ -33,6 +33,59 @@ template <typename real, int DIM> struct MinBlocks {
     static constexpr int value = (sizeof(real) == 4 ? 3 : 2) * 256 / BlockOf<real, DIM>::value;
 };
 
+// ------------------------------------------------- a tile by several CTAs
+//
+// A grid of few tiles leaves most SMs idle at one CTA per tile.  There kSplit
+// CTAs share a tile as a cluster: they take its blocks of records in turn,
+// reserve the slots of the records that stay from one counter (in the first
+// CTA's shared memory), and their current tiles are added word by word over
+// the cluster before they are flushed, so an electron and its ion cancel
+// exactly whichever CTA deposits them.
+constexpr int kSplit = 4;
+
+template <int SPLIT> __device__ __forceinline__ void cluster_sync()
+{
+    if (SPLIT > 1) {
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    } else {
+        __syncthreads();
+    }
+}
+__device__ __forceinline__ unsigned cluster_rank()
+{
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// the address of this CTA's shared variable p in CTA `rank` of the cluster
+__device__ __forceinline__ unsigned cluster_map(const void *p, unsigned rank)
+{
+    unsigned a = (unsigned)__cvta_generic_to_shared(p), d;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(rank));
+    return d;
+}
+__device__ __forceinline__ int cluster_ld(unsigned a, int)
+{
+    int v;
+    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ double cluster_ld(unsigned a, double)
+{
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a));
+    return v;
+}
+// the tile's counter of records that stay: *p of the cluster's first CTA
+template <int SPLIT> __device__ __forceinline__ int stay_add(int *p, int n)
+{
+    if (SPLIT == 1) return atomicAdd(p, n);
+    int old;
+    asm volatile("atom.shared::cluster.add.s32 %0, [%1], %2;" : "=r"(old) : "r"(cluster_map(p, 0)), "r"(n) : "memory");
+    return old;
+}
+
 // ---------------------------------------------------------------- helpers
 
 // Shared-memory current accumulators.  FP32 currents are accumulated exactly,
@@ -212,7 +265,7 @@ __device__ __forceinline__ bool stage_tile(const Geom &g, const Ptr6<real> src, 
 // nodes outside a component's valid z range dropped (absorbing z).  FP32
 // tiles hold fixed-point "hi" and "lo" words (see sh_acc): the node's value is
 // (hi + lo lo_inv) times the component's quantum q_c.
-template <typename real, int DIM, int NC, int QX, int QY, int QZ, int L>
+template <typename real, int DIM, int NC, int QX, int QY, int QZ, int L, int SPLIT>
 __device__ __forceinline__ void flush_tile(const Geom &g, const Ptr3<real> dstJ, unsigned half_z,
                                            const typename Acc<real>::type *src, real q0, real q1, real q2,
                                            real lo_inv, int lox, int loy, int loz)
@@ -220,16 +273,26 @@ __device__ __forceinline__ void flush_tile(const Geom &g, const Ptr3<real> dstJ,
     constexpr int QN = QX * QY * QZ;
     const bool tiny = g.nx < QX || (DIM == 3 && g.ny < QY);
     // each node of the box once, all components of it together
-    for (int r = threadIdx.x; r < QN; r += blockDim.x) {
+    using acc_t = typename Acc<real>::type;
+    // word w of the tile, summed over the cluster (each CTA flushes its share of the nodes)
+    auto word = [&](int w) -> acc_t {
+        if (SPLIT == 1) return src[w];
+        acc_t v = 0;
+#pragma unroll
+        for (unsigned p = 0; p < (unsigned)SPLIT; ++p) v += cluster_ld(cluster_map(src + w, p), acc_t(0));
+        return v;
+    };
+    const int first = (SPLIT > 1 ? (int)(cluster_rank() * blockDim.x) : 0) + (int)threadIdx.x;
+    for (int r = first; r < QN; r += SPLIT * (int)blockDim.x) {
         real v[NC];
         bool any = false;
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
             if constexpr (sizeof(real) == 4) {
-                const int h = src[c * QN + r], l = src[NC * QN + c * QN + r];  // "hi" and "lo" words
+                const int h = word(c * QN + r), l = word(NC * QN + c * QN + r);  // "hi" and "lo" words
                 v[c] = (h | l) == 0 ? real(0) : fmaf((float)l, lo_inv, (float)h);
             } else {
-                v[c] = src[c * QN + r];
+                v[c] = word(c * QN + r);
             }
             any = any || v[c] != real(0);
         }
@@ -863,7 +926,7 @@ __device__ __forceinline__ void ion_deposit(accT *Jz, ar z0, ar z1, ar ox, ar oy
 // (ff) from their stored positions (the end of one step's path is exactly the start of the
 // next one's).  Returns false (nothing done) for an empty bucket.  The loop
 // runs all lanes of a warp (as the electrons', see push_tile).
-template <typename real, int DIM, int S, int TX, int TY, int TZ, int LOFF, bool REL>
+template <typename real, int DIM, int S, int TX, int TY, int TZ, int LOFF, bool REL, int SPLIT>
 __device__ __forceinline__ bool ions_of_tile(const Geom &g, const IonSide<real> &is, int64_t t,
                                              const TilePos<DIM, TX, TY, TZ> &tp, typename Acc<real>::type *Jz,
                                              unsigned char *wbuf, real dz, real scale_z, real lo_scale, unsigned *err,
@@ -901,10 +964,11 @@ __device__ __forceinline__ bool ions_of_tile(const Geom &g, const IonSide<real> 
         at<real>(b, R::W) = w;
         at<int32_t>(ES == 4 ? b : b - (slot & 31) * 4, R::CELL) = cell;
     };
+    const int rank = SPLIT > 1 ? (int)cluster_rank() : 0;
     __syncthreads();
     if (threadIdx.x == 0) *s_stay = 0;
-    __syncthreads();
-    int i = (int)(threadIdx.x >> 5), qn = 0;
+    cluster_sync<SPLIT>();
+    int i = rank * (kBlock / 32) + (int)(threadIdx.x >> 5), qn = 0;
     // the queue's records into the tile below
     auto flush = [&]() {
         __syncwarp();
@@ -935,7 +999,7 @@ __device__ __forceinline__ bool ions_of_tile(const Geom &g, const IonSide<real> 
         real oz = at<real>(rbuf, R::OZ), w = at<real>(rbuf, R::W);
         uint32_t cell = row<uint32_t>(wbuf, R::CELL, lane);
         __syncwarp();
-        i += kBlock / 32;
+        i += SPLIT * (kBlock / 32);
         if (i < bl.n) fetch_block<R::RB>(fbuf, in + (int64_t)bl.block(i) * R::RB, lane);
         int li, lj, lk;
         bool here = tp.local(g, cell, li, lj, lk);
@@ -968,7 +1032,7 @@ __device__ __forceinline__ bool ions_of_tile(const Geom &g, const IonSide<real> 
         cell += (uint32_t)sz << kbit;
         const unsigned ms = __ballot_sync(0xffffffffu, stay), ml = __ballot_sync(0xffffffffu, leave);
         int bs = 0;
-        if (lane == 0) bs = atomicAdd(s_stay, __popc(ms));
+        if (lane == 0) bs = stay_add<SPLIT>(s_stay, __popc(ms));
         bs = __shfl_sync(0xffffffffu, bs, 0) + __popc(ms & lt);
         if (stay) {
             put(out, bs, ox, oy, oz, w, (int32_t)cell);
@@ -992,8 +1056,8 @@ __device__ __forceinline__ bool ions_of_tile(const Geom &g, const IonSide<real> 
         }
     }
     if (qn) flush();
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    cluster_sync<SPLIT>();
+    if (threadIdx.x == 0 && rank == 0) {
         is.out_lo[t] = *s_stay;
         is.in_lo[t] = 0;
         is.in_hi[t] = 0;
@@ -1034,7 +1098,7 @@ __device__ __forceinline__ real rel_step(real dl, real d, int &fold)
 // (33.6M electrons, gamma = 13): half of them still paired 1245 -> 955 us a
 // launch, all paired 703 -> 487 us (58% of the DRAM rate), from 1054M to 702M
 // and 503M to 362M warp instructions.
-template <typename real, int DIM, int S, int TX, int TY, int TZ, bool REL>
+template <typename real, int DIM, int S, int TX, int TY, int TZ, bool REL, int SPLIT = 1>
 __device__ __forceinline__ void push_tile(const PushArgs<real> &a, const int64_t t, unsigned char *smem_raw)
 {
     const Geom &g = a.g;
@@ -1079,8 +1143,9 @@ __device__ __forceinline__ void push_tile(const PushArgs<real> &a, const int64_t
     const int kbit = g.bx + g.by;
     unsigned char *fbuf = wbuf + lane * 16, *rbuf = wbuf + lane * ES;
 
+    const int rank = SPLIT > 1 ? (int)cluster_rank() : 0;
     __syncthreads();  // previous tile finished with shared memory
-    int i = (int)(threadIdx.x >> 5), qn = 0;
+    int i = rank * (kBlock / 32) + (int)(threadIdx.x >> 5), qn = 0;
     if (i < bl.n) fetch_block<R::RB>(fbuf, in + (int64_t)bl.block(i) * R::RB, lane);
     if (threadIdx.x == 0) s_stay = 0;
     // Ez, Bx, By live on half-integer z (bits 2, 3, 4)
@@ -1088,6 +1153,7 @@ __device__ __forceinline__ void push_tile(const PushArgs<real> &a, const int64_t
         g, Ptr6<real>{a.E[0], a.E[1], a.E[2], a.B[0], a.B[1], a.B[2]}, 0x1Cu, sF, tp.lox, tp.loy, tp.loz);
     for (int z = threadIdx.x; z < JB / 16; z += kBlock) reinterpret_cast<int4 *>(sJ)[z] = make_int4(0, 0, 0, 0);
     const bool field_in_tile = __syncthreads_or(staged_nonzero) != 0;
+    if (SPLIT > 1) cluster_sync<SPLIT>();  // the first CTA's counter is set
     bool deposited = false;
 
     // a record into slot s of the bucket at b
@@ -1171,7 +1237,7 @@ __device__ __forceinline__ void push_tile(const PushArgs<real> &a, const int64_t
             if (DIM == 3) dly = at<real>(rbuf, R::DLY);
         }
         __syncwarp();
-        i += kBlock / 32;
+        i += SPLIT * (kBlock / 32);
         if (i < bl.n) fetch_block<R::RB>(fbuf, in + (int64_t)bl.block(i) * R::RB, lane);
         bool paired = (int32_t)word < 0;
         word &= ~kPaired;
@@ -1335,7 +1401,7 @@ __device__ __forceinline__ void push_tile(const PushArgs<real> &a, const int64_t
             const bool stay = valid && in_tile, leave = valid && !in_tile;
             const unsigned ms = __ballot_sync(kAll, stay), ml = __ballot_sync(kAll, leave);
             int bs = 0;
-            if (lane == 0) bs = atomicAdd(&s_stay, __popc(ms));
+            if (lane == 0) bs = stay_add<SPLIT>(&s_stay, __popc(ms));
             bs = __shfl_sync(kAll, bs, 0) + __popc(ms & lt);
             if (stay) {
                 uint32_t nw = word + (uint32_t)mx + ((uint32_t)mz << kbit);
@@ -1427,20 +1493,22 @@ __device__ __forceinline__ void push_tile(const PushArgs<real> &a, const int64_t
         }
     }
     if (qn) flush();
-    deposited = __syncthreads_or(deposited) != 0;
+    deposited = __syncthreads_or(deposited) != 0 || SPLIT > 1;
+    if (SPLIT > 1) cluster_sync<SPLIT>();  // every CTA's records are written
     // the drifting ions of the tile, into the same current tile
     if (a.fuse_ions)
-        deposited |= ions_of_tile<real, DIM, S, TX, TY, TZ, 3 * QN, REL>(g, a.ions, t, tp, sJ + 2 * QN, wbuf, dz_drift,
+        deposited |= ions_of_tile<real, DIM, S, TX, TY, TZ, 3 * QN, REL, SPLIT>(g, a.ions, t, tp, sJ + 2 * QN, wbuf, dz_drift,
                                                                           a.fx_scale[2], a.fx_lo[0], a.err, &s_stay_i);
     // flush the J tile: one global add per non-zero node
     if (deposited)
-        flush_tile<real, DIM, 3, QX, QY, QZ, JL>(g, Ptr3<real>{a.J[0], a.J[1], a.J[2]}, 0x4u, sJ, a.fx_quant[0],
+        flush_tile<real, DIM, 3, QX, QY, QZ, JL, SPLIT>(g, Ptr3<real>{a.J[0], a.J[1], a.J[2]}, 0x4u, sJ, a.fx_quant[0],
                                                  a.fx_quant[1], a.fx_quant[2], a.fx_lo[1], tp.lox, tp.loy, tp.loz);
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && rank == 0) {
         a.out_lo[t] = s_stay;
         a.in_lo[t] = 0;
         a.in_hi[t] = 0;
     }
+    if (SPLIT > 1) cluster_sync<SPLIT>();  // no CTA leaves while another reads its tile
 }
 
 // ------------------------------------------------------ drifting-ion tile
@@ -1467,9 +1535,9 @@ __device__ __forceinline__ void ion_tile(const PushArgs<real> &a, const int64_t 
     const TilePos<DIM, TX, TY, TZ> tp(g, t);
     __syncthreads();
     for (int z = threadIdx.x; z < JB / 16; z += kBlock) reinterpret_cast<int4 *>(sJ)[z] = make_int4(0, 0, 0, 0);
-    ions_of_tile<real, DIM, S, TX, TY, TZ, QN, REL>(g, is, t, tp, sJ, wbuf, dz, a.fx_scale[2], a.fx_lo[0], a.err,
+    ions_of_tile<real, DIM, S, TX, TY, TZ, QN, REL, 1>(g, is, t, tp, sJ, wbuf, dz, a.fx_scale[2], a.fx_lo[0], a.err,
                                                     &s_stay);
-    flush_tile<real, DIM, 1, QX, QY, QZ, JL>(g, Ptr3<real>{a.J[2], a.J[2], a.J[2]}, 0x1u, sJ, a.fx_quant[2],
+    flush_tile<real, DIM, 1, QX, QY, QZ, JL, 1>(g, Ptr3<real>{a.J[2], a.J[2], a.J[2]}, 0x1u, sJ, a.fx_quant[2],
                                              a.fx_quant[2], a.fx_quant[2], a.fx_lo[1], tp.lox, tp.loy, tp.loz);
 }
 
