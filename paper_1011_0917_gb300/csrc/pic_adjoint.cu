@@ -273,6 +273,24 @@ struct Window {
     }
 };
 
+// The windows' x and y lengths the deposit and its transpose go over: a node
+// beyond the support that both ends of every lane's path share (S + 1 nodes)
+// has weight zero, so body(S + 1, S + 1) is enough where no lane of the warp
+// crosses a cell face in x or y, and body(S + 2, S + 2) otherwise (3D CIC: 20
+// and 54 nodes).  In z the drift crosses a face in every warp.  One body per
+// combination of x and y measured no faster (vjp 281 us against 272).
+template <int DIM, int W, typename F>
+__device__ __forceinline__ void for_windows(bool crossed, F body)
+{
+    using wide = std::integral_constant<int, W>;
+    using narrow = std::integral_constant<int, W - 1>;
+    using one = std::integral_constant<int, 1>;
+    using y_wide = typename std::conditional<DIM == 3, wide, one>::type;
+    using y_narrow = typename std::conditional<DIM == 3, narrow, one>::type;
+    if (__any_sync(__activemask(), crossed)) body(wide(), y_wide());
+    else body(narrow(), y_narrow());
+}
+
 }  // namespace
 
 // ------------------------------------------------------------ flat forward
@@ -353,18 +371,24 @@ __device__ __forceinline__ void adj_ion_step(const AdjArgs<real> &a, const Drift
     a.iout.oz[p] = noz;
 }
 
-// resident CTAs of 256 threads the particle kernels are compiled for: in 3D
-// more registers per thread (the windows' 27 nodes) instead of more warps
-template <typename real, int DIM> struct AdjBlocks {
-    static constexpr int push = DIM == 3 ? (sizeof(real) == 4 ? 3 : 2) : 6;
-    static constexpr int vjp = DIM == 3 ? 2 : 3;
+// Resident CTAs of 256 threads the particle kernels are compiled for.  They
+// wait for dependent loads (46% of issue, 25% of L2), so in FP32 more warps pay
+// for some spills: 48 x 48 x 128 cells, 1.2M slots, push with 3 / 4 / 5 / 6
+// CTAs 163 / 143 / 136 / 142 us, vjp with 2 / 3 / 4 / 5 CTAs 302 / 272 / 293 /
+// 349; 2D (128 x 1536) vjp with 3 / 4 / 5 38 / 35 / 35, push no difference
+// from 5 to 8.
+// The quadratic shape's windows (64 nodes) keep fewer CTAs.
+template <typename real, int DIM, int S> struct AdjBlocks {
+    static constexpr bool many = sizeof(real) == 4 && S == 1;
+    static constexpr int push = DIM == 3 ? (many ? 5 : sizeof(real) == 4 ? 3 : 2) : 6;
+    static constexpr int vjp = DIM == 3 ? (many ? 3 : 2) : (many ? 4 : 3);
 };
 
 // One step of the electrons of the flat store: gather E^n, B^n at x^n, Boris,
 // move, Esirkepov deposit with global atomics, re-cell; state `in` -> `out`.
 // Shape order S: supports of S + 1 nodes, Esirkepov windows of W = S + 2.
 template <typename real, int DIM, int S>
-__global__ void __launch_bounds__(256, (AdjBlocks<real, DIM>::push)) adj_push_kernel(AdjArgs<real> a)
+__global__ void __launch_bounds__(256, (AdjBlocks<real, DIM, S>::push)) adj_push_kernel(AdjArgs<real> a)
 {
     chain_begin();
     constexpr int W = S + 2, WY = DIM == 3 ? W : 1;
@@ -404,10 +428,10 @@ __global__ void __launch_bounds__(256, (AdjBlocks<real, DIM>::push)) adj_push_ke
         const real z1 = add_rn(oz, drift.dz) + dvz * a.dtdh[2];
         if (!together) {
             real S0x[W], DSx[W], S0y[W], DSy[W], S0z[W], DSz[W];
-            bool cr;
-            const int ax = ci + esirk_axis_c<S>(ox, x1, S0x, DSx, cr);
-            const int ay = DIM == 3 ? cj + esirk_axis_c<S>(oy, y1, S0y, DSy, cr) : 0;
-            const int az = ck + esirk_axis_c<S>(oz, z1, S0z, DSz, cr);
+            bool crx, cry = false, crz;
+            const int ax = ci + esirk_axis_c<S>(ox, x1, S0x, DSx, crx);
+            const int ay = DIM == 3 ? cj + esirk_axis_c<S>(oy, y1, S0y, DSy, cry) : 0;
+            const int az = ck + esirk_axis_c<S>(oz, z1, S0z, DSz, crz);
             const Window<DIM, W> wn(g, ax, ay, az);
             const real fx = a.jfac[0] * w, fy = a.jfac[1] * w, fz = a.jfac[2] * w, fyv = a.jyfac * w * vy;
             real Rx[W], Ry[W], Rz[W];
@@ -423,35 +447,38 @@ __global__ void __launch_bounds__(256, (AdjBlocks<real, DIM>::push)) adj_push_ke
                     Ry[q] = fy * sy_;
                 }
             }
+            for_windows<DIM, W>(crx || cry, [&](auto nx, auto ny) {
+                constexpr int NX = decltype(nx)::value, NY = decltype(ny)::value;
 #pragma unroll
-            for (int c = 0; c < W; ++c) {
-                const bool in = wn.ok >> c & 1u;
+                for (int c = 0; c < W; ++c) {
+                    const bool in = wn.ok >> c & 1u;
 #pragma unroll
-                for (int b = 0; b < WY; ++b) {  // Jx = fx Rx[q] T(y_b, z_c)
-                    const real T = DIM == 3 ? tshape(S0y[b], DSy[b], S0z[c], DSz[c]) : S0z[c] + real(0.5) * DSz[c];
+                    for (int b = 0; b < NY; ++b) {  // Jx = fx Rx[q] T(y_b, z_c)
+                        const real T = DIM == 3 ? tshape(S0y[b], DSy[b], S0z[c], DSz[c]) : S0z[c] + real(0.5) * DSz[c];
 #pragma unroll
-                    for (int q = 0; q < W - 1; ++q) fadd(a.J[0], wn.z[c] + wn.y[b] + wn.x[q], Rx[q] * T, in);
-                }
+                        for (int q = 0; q < NX - 1; ++q) fadd(a.J[0], wn.z[c] + wn.y[b] + wn.x[q], Rx[q] * T, in);
+                    }
 #pragma unroll
-                for (int q = 0; q < W; ++q) {  // Jy = fy Ry[b] T(z_c, x_q); 2D: fyv T
-                    const real T = tshape(S0z[c], DSz[c], S0x[q], DSx[q]);
-                    if (DIM == 3) {
+                    for (int q = 0; q < NX; ++q) {  // Jy = fy Ry[b] T(z_c, x_q); 2D: fyv T
+                        const real T = tshape(S0z[c], DSz[c], S0x[q], DSx[q]);
+                        if (DIM == 3) {
 #pragma unroll
-                        for (int b = 0; b < W - 1; ++b) fadd(a.J[1], wn.z[c] + wn.y[b] + wn.x[q], Ry[b] * T, in);
-                    } else {
-                        fadd(a.J[1], wn.z[c] + wn.x[q], fyv * T, in);
+                            for (int b = 0; b < NY - 1; ++b) fadd(a.J[1], wn.z[c] + wn.y[b] + wn.x[q], Ry[b] * T, in);
+                        } else {
+                            fadd(a.J[1], wn.z[c] + wn.x[q], fyv * T, in);
+                        }
                     }
                 }
-            }
 #pragma unroll
-            for (int b = 0; b < WY; ++b)
+                for (int b = 0; b < NY; ++b)
 #pragma unroll
-                for (int q = 0; q < W; ++q) {  // Jz = fz Rz[c] T(x_q, y_b)
-                    const real T = DIM == 3 ? tshape(S0x[q], DSx[q], S0y[b], DSy[b]) : S0x[q] + real(0.5) * DSx[q];
+                    for (int q = 0; q < NX; ++q) {  // Jz = fz Rz[c] T(x_q, y_b)
+                        const real T = DIM == 3 ? tshape(S0x[q], DSx[q], S0y[b], DSy[b]) : S0x[q] + real(0.5) * DSx[q];
 #pragma unroll
-                    for (int c = 0; c < W - 1; ++c)
-                        fadd(a.J[2], wn.z[c] + wn.y[b] + wn.x[q], Rz[c] * T, wn.okh >> c & 1u);
-                }
+                        for (int c = 0; c < W - 1; ++c)
+                            fadd(a.J[2], wn.z[c] + wn.y[b] + wn.x[q], Rz[c] * T, wn.okh >> c & 1u);
+                    }
+            });
         }
         // new cell (an offset that rounds to 1 moves on)
         int sx = (int)floor(x1), sy = DIM == 3 ? (int)floor(y1) : 0, sz = (int)floor(z1);
@@ -533,7 +560,7 @@ __device__ __forceinline__ real adj_ion_vjp_one(const AdjArgs<real> &a, const Dr
 // du^{n-1/2} in their place, adds the gather's field cotangents to lE, lB and
 // the weight's cotangent to lw.
 template <typename real, int DIM, int S>
-__global__ void __launch_bounds__(256, (AdjBlocks<real, DIM>::vjp)) adj_push_vjp_kernel(AdjArgs<real> a)
+__global__ void __launch_bounds__(256, (AdjBlocks<real, DIM, S>::vjp)) adj_push_vjp_kernel(AdjArgs<real> a)
 {
     chain_begin();
     constexpr int W = S + 2, WY = DIM == 3 ? W : 1;
@@ -581,7 +608,7 @@ __global__ void __launch_bounds__(256, (AdjBlocks<real, DIM>::vjp)) adj_push_vjp
             S0y[q] = real(q == 0);
             DSy[q] = real(0);
         }
-        bool cr;
+        bool crx, cry = false, crz;
         real wtmp[S + 1], dw0x[S + 1], dw1x[S + 1], dw0y[S + 1], dw1y[S + 1], dw0z[S + 1], dw1z[S + 1];
         const int b0x = offset_weights<S>(ox, wtmp), b1x = spline_weights<S>(x1, wtmp);
         const int b0z = offset_weights<S>(oz, wtmp), b1z = spline_weights<S>(z1, wtmp);
@@ -589,15 +616,15 @@ __global__ void __launch_bounds__(256, (AdjBlocks<real, DIM>::vjp)) adj_push_vjp
         spline_dw<S>(x1, dw1x);
         spline_dw<S>(oz, dw0z);
         spline_dw<S>(z1, dw1z);
-        const int anx = esirk_axis_c<S>(ox, x1, S0x, DSx, cr);
-        const int anz = esirk_axis_c<S>(oz, z1, S0z, DSz, cr);
+        const int anx = esirk_axis_c<S>(ox, x1, S0x, DSx, crx);
+        const int anz = esirk_axis_c<S>(oz, z1, S0z, DSz, crz);
         int b0y = 0, b1y = 0, any_ = 0;
         if (DIM == 3) {
             b0y = offset_weights<S>(oy, wtmp);
             b1y = spline_weights<S>(y1, wtmp);
             spline_dw<S>(oy, dw0y);
             spline_dw<S>(y1, dw1y);
-            any_ = esirk_axis_c<S>(oy, y1, S0y, DSy, cr);
+            any_ = esirk_axis_c<S>(oy, y1, S0y, DSy, cry);
         }
         const int ax = ci + anx, ay = cj + any_, az = ck + anz;
         real Rx[W], Ry[W], Rz[W];
@@ -626,93 +653,96 @@ __global__ void __launch_bounds__(256, (AdjBlocks<real, DIM>::vjp)) adj_push_vjp
         auto dT1 = [&](real s0v, real dsv) { return half * s0v + third * dsv; };
         const Window<DIM, W> wn(g, ax, ay, az);
         if (a.lj_plane[ck]) {  // (else every current cotangent in reach is zero)
-            const real *J0 = a.J[0], *J1 = a.J[1], *J2 = a.J[2];
-            real gT, lw = 0;
-            // Jx = fx Rx[q] T(y_b, z_c)
+            for_windows<DIM, W>(crx || cry, [&](auto nx, auto ny) {
+                constexpr int NX = decltype(nx)::value, NY = decltype(ny)::value;
+                const real *J0 = a.J[0], *J1 = a.J[1], *J2 = a.J[2];
+                real gT, lw = 0;
+                // Jx = fx Rx[q] T(y_b, z_c)
 #pragma unroll
-            for (int c = 0; c < W; ++c) {
-                const bool in = wn.ok >> c & 1u;
+                for (int c = 0; c < W; ++c) {
+                    const bool in = wn.ok >> c & 1u;
 #pragma unroll
-                for (int b = 0; b < WY; ++b) {
-                    const real T = tshape(S0y[b], DSy[b], S0z[c], DSz[c]);
-                    gT = 0;
+                    for (int b = 0; b < NY; ++b) {
+                        const real T = tshape(S0y[b], DSy[b], S0z[c], DSz[c]);
+                        gT = 0;
 #pragma unroll
-                    for (int q = 0; q < W - 1; ++q) {
-                        const real l = in ? J0[wn.z[c] + wn.y[b] + wn.x[q]] : real(0);
-                        gRx[q] += T * l;
-                        gT += Rx[q] * l;
-                    }
-                    lw += gT * T;
-                    gT *= fx;
-                    gS0z[c] += gT * dT0(S0y[b], DSy[b]);
-                    gDSz[c] += gT * dT1(S0y[b], DSy[b]);
-                    if (DIM == 3) {
-                        gS0y[b] += gT * dT0(S0z[c], DSz[c]);
-                        gDSy[b] += gT * dT1(S0z[c], DSz[c]);
-                    }
-                }
-            }
-            Lw += a.jfac[0] * lw;
-            lw = 0;
-            // Jy = fy Ry[b] T(z_c, x_q); 2D out of plane: Jy = fy1 w T(x_q, z_c)
-#pragma unroll
-            for (int c = 0; c < W; ++c) {
-                const bool in = wn.ok >> c & 1u;
-#pragma unroll
-                for (int q = 0; q < W; ++q) {
-                    const real T = tshape(S0z[c], DSz[c], S0x[q], DSx[q]);
-                    gT = 0;
-                    if (DIM == 3) {
-#pragma unroll
-                        for (int b = 0; b < W - 1; ++b) {
-                            const real l = in ? J1[wn.z[c] + wn.y[b] + wn.x[q]] : real(0);
-                            gRy[b] += T * l;
-                            gT += Ry[b] * l;
+                        for (int q = 0; q < NX - 1; ++q) {
+                            const real l = in ? J0[wn.z[c] + wn.y[b] + wn.x[q]] : real(0);
+                            gRx[q] += T * l;
+                            gT += Rx[q] * l;
                         }
                         lw += gT * T;
-                        gT *= fy;
-                    } else {
-                        const real l = in ? J1[wn.z[c] + wn.x[q]] : real(0);
-                        Ly += T * l;
-                        gT = fy1 * w * l;
+                        gT *= fx;
+                        gS0z[c] += gT * dT0(S0y[b], DSy[b]);
+                        gDSz[c] += gT * dT1(S0y[b], DSy[b]);
+                        if (DIM == 3) {
+                            gS0y[b] += gT * dT0(S0z[c], DSz[c]);
+                            gDSy[b] += gT * dT1(S0z[c], DSz[c]);
+                        }
                     }
-                    gS0z[c] += gT * dT0(S0x[q], DSx[q]);
-                    gDSz[c] += gT * dT1(S0x[q], DSx[q]);
-                    gS0x[q] += gT * dT0(S0z[c], DSz[c]);
-                    gDSx[q] += gT * dT1(S0z[c], DSz[c]);
                 }
-            }
-            if (DIM == 3) Lw += a.jfac[1] * lw;
-            lw = 0;
-            // Jz = fz Rz[c] T(x_q, y_b)
+                Lw += a.jfac[0] * lw;
+                lw = 0;
+                // Jy = fy Ry[b] T(z_c, x_q); 2D out of plane: Jy = fy1 w T(x_q, z_c)
 #pragma unroll
-            for (int b = 0; b < WY; ++b)
+                for (int c = 0; c < W; ++c) {
+                    const bool in = wn.ok >> c & 1u;
+#pragma unroll
+                    for (int q = 0; q < NX; ++q) {
+                        const real T = tshape(S0z[c], DSz[c], S0x[q], DSx[q]);
+                        gT = 0;
+                        if (DIM == 3) {
+#pragma unroll
+                            for (int b = 0; b < NY - 1; ++b) {
+                                const real l = in ? J1[wn.z[c] + wn.y[b] + wn.x[q]] : real(0);
+                                gRy[b] += T * l;
+                                gT += Ry[b] * l;
+                            }
+                            lw += gT * T;
+                            gT *= fy;
+                        } else {
+                            const real l = in ? J1[wn.z[c] + wn.x[q]] : real(0);
+                            Ly += T * l;
+                            gT = fy1 * w * l;
+                        }
+                        gS0z[c] += gT * dT0(S0x[q], DSx[q]);
+                        gDSz[c] += gT * dT1(S0x[q], DSx[q]);
+                        gS0x[q] += gT * dT0(S0z[c], DSz[c]);
+                        gDSx[q] += gT * dT1(S0z[c], DSz[c]);
+                    }
+                }
+                if (DIM == 3) Lw += a.jfac[1] * lw;
+                lw = 0;
+                // Jz = fz Rz[c] T(x_q, y_b)
+#pragma unroll
+                for (int b = 0; b < NY; ++b)
+#pragma unroll
+                    for (int q = 0; q < NX; ++q) {
+                        const real T = tshape(S0x[q], DSx[q], S0y[b], DSy[b]);
+                        gT = 0;
+#pragma unroll
+                        for (int c = 0; c < W - 1; ++c) {
+                            const real l = wn.okh >> c & 1u ? J2[wn.z[c] + wn.y[b] + wn.x[q]] : real(0);
+                            gRz[c] += T * l;
+                            gT += Rz[c] * l;
+                        }
+                        lw += gT * T;
+                        gT *= fz;
+                        gS0x[q] += gT * dT0(S0y[b], DSy[b]);
+                        gDSx[q] += gT * dT1(S0y[b], DSy[b]);
+                        if (DIM == 3) {
+                            gS0y[b] += gT * dT0(S0x[q], DSx[q]);
+                            gDSy[b] += gT * dT1(S0x[q], DSx[q]);
+                        }
+                    }
+                Lw += a.jfac[2] * lw;
 #pragma unroll
                 for (int q = 0; q < W; ++q) {
-                    const real T = tshape(S0x[q], DSx[q], S0y[b], DSy[b]);
-                    gT = 0;
-#pragma unroll
-                    for (int c = 0; c < W - 1; ++c) {
-                        const real l = wn.okh >> c & 1u ? J2[wn.z[c] + wn.y[b] + wn.x[q]] : real(0);
-                        gRz[c] += T * l;
-                        gT += Rz[c] * l;
-                    }
-                    lw += gT * T;
-                    gT *= fz;
-                    gS0x[q] += gT * dT0(S0y[b], DSy[b]);
-                    gDSx[q] += gT * dT1(S0y[b], DSy[b]);
-                    if (DIM == 3) {
-                        gS0y[b] += gT * dT0(S0x[q], DSx[q]);
-                        gDSy[b] += gT * dT1(S0x[q], DSx[q]);
-                    }
+                    gRx[q] *= fx;
+                    gRy[q] *= fy;
+                    gRz[q] *= fz;
                 }
-            Lw += a.jfac[2] * lw;
-#pragma unroll
-            for (int q = 0; q < W; ++q) {
-                gRx[q] *= fx;
-                gRy[q] *= fy;
-                gRz[q] *= fz;
-            }
+            });
         }
         if (DIM == 2) Lw += fy1 * Ly;
         // running sums: R[q] = sum_{q' <= q} DS[q']
