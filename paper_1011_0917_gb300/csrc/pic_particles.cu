@@ -46,14 +46,17 @@ static void launch_push_z(const PushArgs<real> &a, bool ions, cudaStream_t s)
     const size_t smem = push_smem<real, DIM, S, TX, TY, TZ, REL>(ions);
     auto k = ions ? ion_kernel<real, DIM, S, TX, TY, TZ, REL> : push_kernel<real, DIM, S, TX, TY, TZ, REL>;
     if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    // one CTA per tile, or kSplit where those of all tiles are resident at once
-    // (the default tile shapes): beyond that the CTAs of one tile each already
-    // fill the device.  A pass of 16 steps on 64 x 512 cells (128 tiles) 784 ->
-    // 581 us, 4 steps on 64 x 256 in FP64 (64 tiles of 900 particles) 1083 ->
-    // 824 us.
+    // One CTA per tile, or kSplit (the default tile shapes) where the tiles are
+    // fewer than the SMs or kSplit CTAs for each are resident at once; beyond
+    // that the tiles fill the device and splitting them repeats their staging.
+    // us per pass, one CTA / kSplit: 64 x 512 cells (128 tiles, 16 steps) 784 /
+    // 581; FP64, 4 steps, 900 particles a tile: 64 tiles 1083 / 824, 96 tiles
+    // 1488 / 1067, 152 tiles 1069 / 1293; 3D: 125 tiles 416 / 395, 432 tiles
+    // 500 / 581; 2D: 304 tiles 693 / 705.
     constexpr bool kDefaultTile = DIM == 3 ? TZ == 8 : TX == 16;
     if constexpr (kDefaultTile) {
-        if (!ions && a.g.ntiles * kSplit <= (int64_t)device_sms() * MinBlocks<real, DIM>::value) {
+        const int64_t sms = device_sms();
+        if (!ions && (a.g.ntiles < sms || a.g.ntiles * kSplit <= sms * MinBlocks<real, DIM>::value)) {
             auto ks = push_split_kernel<real, DIM, S, TX, TY, TZ, REL>;
             if (smem > 48 * 1024) cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             launch_clusters(chained(a.g), kSplit, ks, (unsigned)(a.g.ntiles * kSplit), BlockOf<real, DIM>::value, smem, s, a);

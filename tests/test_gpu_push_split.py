@@ -10,12 +10,13 @@ from test_gpu_push_blocks import FP32, FP64, O, test_leavers_of_one_tile as leav
 
 pytestmark = pytest.mark.gpu
 
-# tiles: 2D 16 x 16 cells, 3D 8 x 8 x 8; (240, 240) and (64, 40, 48) are just
-# under or above the line on devices of 148 to 160 SMs
+# tiles: 2D 16 x 16 cells, 3D 8 x 8 x 8: 56 and 289, 36, 144 and 180 (152 SMs:
+# the line is at 228 tiles in 2D FP32 and at 152 otherwise)
 GRIDS = [dict(dim=2, nx=112, nz=128, dx=1.0, dz=1.0, filter_passes=1, seed=3),
          dict(dim=2, nx=272, nz=272, dx=1.0, dz=1.0, filter_passes=1, seed=3),
          dict(dim=3, nx=24, ny=24, nz=32, dx=1.0, dy=1.0, dz=1.0, filter_passes=1, seed=4),
-         dict(dim=3, nx=48, ny=48, nz=32, dx=1.0, dy=1.0, dz=1.0, filter_passes=1, seed=4)]
+         dict(dim=3, nx=48, ny=48, nz=32, dx=1.0, dy=1.0, dz=1.0, filter_passes=1, seed=4),
+         dict(dim=3, nx=48, ny=48, nz=40, dx=1.0, dy=1.0, dz=1.0, filter_passes=1, seed=4)]
 
 
 @pytest.mark.parametrize("prec", [FP32, FP64])
