@@ -386,9 +386,8 @@ pic_status pic_batch_set_graph(pic_batch *batch, int steps_per_graph);
    zeroing of the raw currents, the particle push -- a persistent grid whose
    CTAs take (run, tile) items from a device-wide counter, so runs of uneven
    size share the GPU to the last tile -- the drifting ions, the antenna,
-   the filter (3D runs take the plane-load filter instead of the TMA one: a
-   tensor map is made per launch), the Yee update and the injection.  Chains
-   overlap one chain's field phases with another's push.  Each item is
+   the filter, the Yee update and the injection.  Chains overlap one chain's
+   field phases with another's push.  Each item is
    processed by the same code and arithmetic as in a single run's launch, so
    the results are those of the per-context graph (up to the order of the
    floating-point additions of tiles into J).  fused = 0: the per-context
