@@ -48,14 +48,25 @@ static unsigned grid_for(int64_t n, int block)
 constexpr int kAhead = 3;
 __device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
+// Longest chunk of the 3D marches.  The columns next to each other share their
+// halo through the L2 only while they are at about the same plane; in longer
+// chunks they drift apart.  256 x 256 x 512 nodes, chunks as the waves alone
+// would have them (103 planes) / at most 64 / 32 / 16: Yee 456 / 436 / 435 /
+// 441 us, filter (2 passes) 324 / 271 / 268 / 295.
+constexpr int kChunk3 = 32;
+
 // Planes per chunk of a march over nzo planes in ncol columns, each chunk
 // walking `halo` planes more than its own and `resident` chunks running at a
 // time: the length that makes the number of waves times a wave's length
-// smallest (at least cmin planes).
-static int chunk_planes(int64_t nzo, int64_t ncol, int64_t resident, int halo, int cmin)
+// smallest (at least cmin planes, about cmax at most where cmax > 0).
+static int chunk_planes(int64_t nzo, int64_t ncol, int64_t resident, int halo, int cmin, int cmax = 0)
 {
-    const int64_t m0 = (ncol + resident - 1) / resident;
-    int64_t best = nzo, cost = INT64_MAX;
+    int64_t m0 = (ncol + resident - 1) / resident;
+    if (cmax > 0) {
+        const int64_t need = ((nzo + cmax - 1) / cmax * ncol + resident - 1) / resident;
+        if (need > m0) m0 = need;
+    }
+    int64_t best = cmax > 0 && cmax < nzo ? cmax : nzo, cost = INT64_MAX;
     for (int64_t m = m0; m < m0 + 16; ++m) {
         const int64_t chunks = m * resident / ncol;
         if (chunks < 1) continue;
@@ -724,7 +735,7 @@ void launch_yee(const Geom &g, real *const F[9], real *const F1[6], double dt, d
     }
     {
         const int64_t ncol = (int64_t)((g.nx + kColOwn - 1) / kColOwn) * ((g.ny + kCol3Y - 1) / kCol3Y);
-        a.cz = chunk_planes(nzo, ncol * batch_runs(), (int64_t)device_sms() * 2, 3, 4);
+        a.cz = chunk_planes(nzo, ncol * batch_runs(), (int64_t)device_sms() * 2, 3, 4, kChunk3);
         a.nchunks = (nzo + a.cz - 1) / a.cz;
         const int64_t nblocks = ncol * a.nchunks;
         if (record_launch(kBPYee, launch_yee3d_batch<real>, a, nblocks)) return;
@@ -1161,7 +1172,7 @@ static void launch_march(const Geom &g, const real *in, real *out, cudaStream_t 
         constexpr int OWN = 32 - 2 * H;
         const int64_t ncol = (int64_t)((g.nx + OWN - 1) / OWN) * ((g.ny + OWN - 1) / OWN);
         const int cz = chunk_planes(nzo, ncol * batch_runs(), (int64_t)device_sms() * (sizeof(real) == 4 && H <= 2 ? 2 : 1),
-                                    2 * H, 4);
+                                    2 * H, 4, kChunk3);
         const int nchunks = (nzo + cz - 1) / cz;
         const int64_t nblocks = ncol * nchunks;
         if (record_launch(kBPFilter, launch_filter3d_batch<real, H>, MarchArgs<real>{g, in, out, cz, nchunks},
