@@ -542,8 +542,11 @@ pic_status pic_state_bytes(pic_ctx *ctx, size_t *bytes);
    smaller than pic_state_bytes). */
 pic_status pic_get_state(pic_ctx *ctx, void *dst, size_t dst_bytes, int dst_is_device);
 
-/* Restores a snapshot taken from a context with the same grid parameters.
-   PIC_ERR_ARG if it does not match; PIC_ERR_CAPACITY on bucket overflow. */
+/* Restores a snapshot taken from a context with the same grid parameters, from
+   host memory or (src_is_device) the memory of any device a copy can reach:
+   it is read in place on the context's own device and in managed memory, and
+   copied to the context's device first from elsewhere.  PIC_ERR_ARG if it does
+   not match; PIC_ERR_CAPACITY on bucket overflow. */
 pic_status pic_set_state(pic_ctx *ctx, const void *src, size_t src_bytes, int src_is_device);
 
 /* ------------------------------------------------------------- cell order */

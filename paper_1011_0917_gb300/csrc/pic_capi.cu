@@ -88,6 +88,7 @@ struct pic_ctx {
     bool ions_species = false;
     bool rel = false;  // electron records in relative form (rel_actual)
     int sms = 152;     // multiprocessors of the device the buffers live on (set at binding)
+    int device = -1;   // that device (-1: unknown)
 
     size_t field_bytes = 0, species_bytes[2] = {0, 0}, scratch_bytes = 0;
     int64_t slots = 0;
@@ -478,8 +479,10 @@ extern "C" pic_status pic_bind_buffers(pic_ctx *c, const pic_buffers *b)
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0)
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0) {
         c->sms = n;
+        c->device = dev;
+    }
     c->fset = 0;
     c->bound = true;
     return PIC_OK;
@@ -641,8 +644,21 @@ static pic_status bucket_flat(pic_ctx *c, int sp, int64_t n, const Species<real>
     return check_device_error(c);
 }
 
-// bucket flat columns: from where they are when the device can read them
-// there, else through a copy in the staging (inactive) side
+// Can the context's kernels read p where it is?  Memory of its own device and
+// managed memory; another device's may be out of its kernels' reach, which
+// copies are not.
+static bool in_reach(const pic_ctx *c, const void *p)
+{
+    cudaPointerAttributes a{};
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();  // (not an error of the call)
+        return false;
+    }
+    return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == c->device);
+}
+
+// bucket flat columns: from where they are when the context's device can read
+// them there, else through a copy in the staging (inactive) side
 template <typename real>
 static pic_status upload_flat(pic_ctx *c, int sp, int64_t n, const void *const cols[kAttrs], int src_is_device)
 {
@@ -651,7 +667,7 @@ static pic_status upload_flat(pic_ctx *c, int sp, int64_t n, const void *const c
     for (int a = 0; a < kAttrs; ++a) {
         if (c->side[sp].off[a] == SIZE_MAX) continue;
         own[a] = const_cast<void *>(cols[a]);
-        direct = direct && cols[a] && (uintptr_t)cols[a] % attr_size(c, a) == 0;
+        direct = direct && cols[a] && (uintptr_t)cols[a] % attr_size(c, a) == 0 && in_reach(c, cols[a]);
     }
     if (direct) return bucket_flat<real>(c, sp, n, view_of<real>(own, 32, 32));
     void *dst[kAttrs];
