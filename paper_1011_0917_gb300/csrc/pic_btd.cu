@@ -78,7 +78,9 @@ template void launch_btd<double>(const BtdArgs<double> &, cudaStream_t);
 // gam (f + sgn beta (p0 + p1) / 2), rounded once to the working precision:
 // FP64 in FP64, pairs of FP32 words (about 46 bits) in FP32, where the FP64
 // pipe bounded it (1.2M nodes, six components: 6 launches of 17.6 us; one
-// launch of 35 us with the pairs, 1.7 TB/s: 5.8 us a component)
+// launch of 35 us with the pairs, 1.7 TB/s: 5.8 us a component).  The pairs'
+// error words turn an infinite term into NaN, so what does not come out finite
+// is taken in FP64 again.
 __device__ __forceinline__ double lab_value(double f, double p0, double p1, double gam, double sb)
 {
     return gam * (f + sb * (0.5 * (p0 + p1)));
@@ -104,7 +106,8 @@ __global__ void lab_fields_kernel(LabArgs<real> a)
     real *out = a.out[blockIdx.y];
     const bool half = comp == 2 || comp == 3 || comp == 4;
     const int km = zmax_of(g, half), kmp = zmax_of(g, !half);  // its range, its partner's
-    const T gam(a.gam), sb(comp == 1 || comp == 3 ? -a.beta : a.beta);
+    const double sbeta = comp == 1 || comp == 3 ? -a.beta : a.beta;
+    const T gam(a.gam), sb(sbeta);
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < g.ncomp; r += (int64_t)gridDim.x * blockDim.x) {
         const int k = g.ncomp <= 0x7fffffffLL ? (int)((unsigned)r / (unsigned)g.plane) : (int)(r / g.plane);
         real v = real(0);
@@ -120,7 +123,9 @@ __global__ void lab_fields_kernel(LabArgs<real> a)
                     if (hi > kmp) hi = lo;
                     if (lo > kmp) lo = hi = kmp;
                 }
-                v = lab_value(v, P[r + (lo - k) * g.plane], P[r + (hi - k) * g.plane], gam, sb);
+                const real f = v, p0 = P[r + (lo - k) * g.plane], p1 = P[r + (hi - k) * g.plane];
+                v = lab_value(f, p0, p1, gam, sb);
+                if (sizeof(real) == 4 && !isfinite(v)) v = (real)lab_value((double)f, (double)p0, (double)p1, a.gam, sbeta);
             }
         }
         out[r] = v;
