@@ -2018,7 +2018,7 @@ static pic_status diagnostics_t(pic_ctx *c, pic_diag *out)
     for (int sp = 0; sp < nsp; ++sp) {
         nb[sp] = launch_particle_sums<real>(c->g, species_view<real>(c, sp, c->cur[sp]), counts(c, sp, c->cur[sp], 0),
                                             counts(c, sp, c->cur[sp], 1), sp == 0 ? -1.0 : 1.0, drift_u<real>(c),
-                                            part + used, kPartialBlocks, c->stream);
+                                            c->wmax, part + used, kPartialBlocks, c->stream);
         used += (size_t)4 * nb[sp];
     }
     CUDA_TRY(c, cudaGetLastError());

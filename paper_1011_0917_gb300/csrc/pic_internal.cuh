@@ -867,7 +867,7 @@ void launch_rho(const Geom &g, const Species<real> &sp, const int *lo, const int
                 cudaStream_t s);
 template <typename real>
 int launch_particle_sums(const Geom &g, const Species<real> &sp, const int *lo, const int *hi, double q,
-                          real u_drift, double *partials, int max_blocks, cudaStream_t s);
+                          real u_drift, double wmax, double *partials, int max_blocks, cudaStream_t s);
 void launch_inject(const InjectArgs &a, cudaStream_t s);
 template <typename real>
 void launch_btd(const BtdArgs<real> &a, cudaStream_t s);

@@ -445,9 +445,11 @@ void launch_rho(const Geom &g, const Species<real> &sp, const int *lo, const int
 // reached, most of a boosted plasma) share one gamma - 1, rest_ke: only their
 // weights are summed.  (256 x 8192 cells, 8.4M electrons, 6% of them moving: 324 us
 // per species with the FP64 kinetic energy of every record.)
+// run_len: records whose weights a thread adds between two flushes, at most
+// kSumRun (fewer for weights whose sums would leave the FP32 range)
 template <typename real>
 __global__ void particle_sums_kernel(Geom g, Species<real> sp, const int *lo, const int *hi, double q, double iuz,
-                                     double rest_ke, double *partials)
+                                     double rest_ke, int run_len, double *partials)
 {
     RunSum<real> rest, charge;
     Kahan moving;
@@ -480,7 +482,7 @@ __global__ void particle_sums_kernel(Geom g, Species<real> sp, const int *lo, co
                 const double u2 = vx * vx + vy * vy + vz * vz;
                 moving.add((double)w * (u2 / (sqrt(1.0 + u2) + 1.0)));  // gamma - 1 without cancellation
             }
-            if (++run == kSumRun) {
+            if (++run == run_len) {
                 rest.flush();
                 charge.flush();
                 run = 0;
@@ -516,13 +518,13 @@ __global__ void particle_sums_kernel(Geom g, Species<real> sp, const int *lo, co
 // (an idle block costs FP64 additions too)
 template <typename real>
 int launch_particle_sums(const Geom &g, const Species<real> &sp, const int *lo, const int *hi, double q, real u_drift,
-                         double *partials, int max_blocks, cudaStream_t s)
+                         double wmax, double *partials, int max_blocks, cudaStream_t s)
 {
     const int64_t cap = std::min<int64_t>(max_blocks, (int64_t)device_sms() * 4);
     const int nblocks = (int)std::min(cap, g.ntiles);
     const double u = (double)u_drift;
     particle_sums_kernel<real><<<nblocks, 256, 0, s>>>(g, sp, lo, hi, q, u, u * u / (std::sqrt(1.0 + u * u) + 1.0),
-                                                       partials);
+                                                       wmax * kSumRun < 1e38 ? kSumRun : 1, partials);
     return nblocks;
 }
 
@@ -537,7 +539,7 @@ int launch_particle_sums(const Geom &g, const Species<real> &sp, const int *lo, 
     template void launch_rho<real>(const Geom &, const Species<real> &, const int *, const int *, real, \
                                    real *, cudaStream_t);                                            \
     template int launch_particle_sums<real>(const Geom &, const Species<real> &, const int *,      \
-                                             const int *, double, real, double *, int,      \
+                                             const int *, double, real, double, double *, int, \
                                              cudaStream_t);
 PIC_INSTANTIATE(float)
 PIC_INSTANTIATE(double)

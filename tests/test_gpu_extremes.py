@@ -1,6 +1,8 @@
 """Values at the ends of the working precision in the calls that read results:
 infinities, NaN and values whose sums leave the range in the lab-frame view,
-against the same formulas in FP64 rounded once."""
+weights whose sums leave it in the diagnostics, against FP64."""
+import math
+
 import numpy as np
 import pytest
 
@@ -62,3 +64,28 @@ def test_lab_view_of_extreme_fields(dim, gam, prec):
                 assert (np.abs(g.astype(np.float64) - want)[finite] <= bound[finite]).all(), c
         for c in ("Ez", "Bz"):
             assert np.array_equal(got[c], F[c], equal_nan=True), c
+
+
+@pytest.mark.parametrize("prec", [FP32, FP64])
+@pytest.mark.parametrize("w", [1e29, 3e30, 3e38])
+def test_sums_of_huge_weights(w, prec):
+    # 3000 records in one tile, half of them at rest relative to the drift: a
+    # thread adds a dozen of them before its sum is carried over to FP64
+    import paper_1011_0917_gb300 as P
+    sim = P.Simulation(dim=2, nx=16, nz=16, dx=1.0, dz=0.1, gamma_boost=5.0, precision=prec, slots_per_cell=16.0)
+    real = np.float32 if prec == FP32 else np.float64
+    rng = np.random.default_rng(2)
+    n = 3000
+    U = float(real(-5.0 * sim.sizes.beta))
+    st = np.zeros((7, n))
+    st[0], st[2] = rng.uniform(0.0, 16.0, n), rng.uniform(0.0, 15.9, n) * sim.sizes.hz
+    st[3, ::2] = rng.normal(size=n // 2).astype(np.float32)
+    st[5] = U
+    st[6] = (w * rng.uniform(0.5, 1.0, n)).astype(real)
+    sim.load_particles(0, st)
+    d = sim.diagnostics()
+    want = math.fsum(st[6])
+    assert abs(d.charge + want) <= 1e-15 * want
+    u2 = np.longdouble(st[3]) ** 2 + np.longdouble(U) ** 2
+    want = float(np.sum(np.longdouble(st[6]) * (u2 / (np.sqrt(1 + u2) + 1))))
+    assert abs(d.kinetic_energy - want) <= 1e-15 * want
