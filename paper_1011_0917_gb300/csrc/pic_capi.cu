@@ -1027,8 +1027,7 @@ static void run_phases_t(pic_ctx *c, unsigned mask)
         for (int q = 0; q < 3; ++q) R[q] = tmp + (size_t)q * c->g.ncomp;
     if (mask & PIC_PH_ZERO_J) {
         PhaseTimer pt(c, 0);
-        launch_zero<real>(R[0], (int64_t)3 * c->g.ncomp, c->stream);
-        c->kernels += 1;
+        c->kernels += launch_zero<real>(R[0], (int64_t)3 * c->g.ncomp, c->stream);
     }
     // With ions paired to their electrons, the electron kernel also takes the
     // tile's drifting ion records, so electron and ion currents add in one

@@ -1344,26 +1344,28 @@ __global__ void __launch_bounds__(256) zero_kernel(real *p, int64_t n, unsigned 
     for (int64_t o = first; o < m; o += stride) q[o] = 0;
 }
 
+// returns the kernels it launches
 template <typename real>
-static void zero_launch(real *p, int64_t n, unsigned char *q, int64_t m, cudaStream_t s)
+static int zero_launch(real *p, int64_t n, unsigned char *q, int64_t m, cudaStream_t s)
 {
     // a large array, or one off the 16-byte grid (J of an odd grid, zeroed
     // by itself): a plain memset
     if (n > 3 * kChainNodes || reinterpret_cast<uintptr_t>(p) % 16 != 0) {
         cudaMemsetAsync(p, 0, (size_t)n * sizeof(real), s);
         n = 0;
-        if (m == 0) return;
+        if (m == 0) return 0;
     }
     launch_chained(true, zero_kernel<real>, grid_for(n / 4 + 1, 256), 256, 0, s, p, n, q, m);
+    return 1;
 }
 
 template <typename real>
-void launch_zero(real *p, int64_t n, cudaStream_t s)
+int launch_zero(real *p, int64_t n, cudaStream_t s)
 {
-    if (n <= 0) return;
+    if (n <= 0) return 0;
     if (record_launch(kBPZero, launch_zero_batch<real>, ZeroArgs<real>{p, n}, (n + kZeroChunk - 1) / kZeroChunk))
-        return;
-    zero_launch(p, n, nullptr, 0, s);
+        return 1;
+    return zero_launch(p, n, nullptr, 0, s);
 }
 
 template <typename real>
@@ -1439,7 +1441,7 @@ int launch_field_sums(const Geom &g, real *const F[9], double *partials, int max
     template void launch_antenna<real>(const Geom &, real *, int, int, double, double, double, double,  \
                                        double, double, cudaStream_t, const double *);                   \
     template int launch_field_sums<real>(const Geom &, real *const[9], double *, int, cudaStream_t); \
-    template void launch_zero<real>(real *, int64_t, cudaStream_t);                                     \
+    template int launch_zero<real>(real *, int64_t, cudaStream_t);                                      \
     template void launch_zero2<real>(real *, int64_t, unsigned char *, int64_t, cudaStream_t);
 PIC_FIELDS_INSTANTIATE(float)
 PIC_FIELDS_INSTANTIATE(double)

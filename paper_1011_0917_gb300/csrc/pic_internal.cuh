@@ -850,7 +850,8 @@ struct ZeroArgs {
     real *p;
     int64_t n;
 };
-template <typename real> void launch_zero(real *p, int64_t n, cudaStream_t s);
+// (returns the kernels it launches: none where a memset does it)
+template <typename real> int launch_zero(real *p, int64_t n, cudaStream_t s);
 // the same for two arrays in one launch (q: m bytes)
 template <typename real> void launch_zero2(real *p, int64_t n, unsigned char *q, int64_t m, cudaStream_t s);
 // SMs of the current device (cached per device)
