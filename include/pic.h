@@ -47,7 +47,7 @@ typedef enum pic_status {
     PIC_ERR_CAPACITY = 4, /* a tile bucket overflowed; particles were dropped  */
     PIC_ERR_CFL = 5,      /* a particle moved a cell or more in one step       */
     PIC_ERR_NAN = 6,      /* a non-finite momentum or position was produced    */
-    PIC_ERR_TIMEOUT = 7   /* reserved for bounded device waits                 */
+    PIC_ERR_TIMEOUT = 7   /* pic_wait_check: the bounded wait ran out           */
 } pic_status;
 
 enum { PIC_BC_PERIODIC = 0, PIC_BC_MUR = 1 };       /* z boundary (x, y periodic) */
@@ -256,7 +256,7 @@ pic_status pic_launch_laser(pic_ctx *ctx, const pic_laser_params *p);
 /* ------------------------------------------------------------------ step */
 
 /* Advances nsteps full steps, synchronises the stream and checks the device
-   error word (PIC_ERR_CAPACITY / PIC_ERR_CFL / PIC_ERR_NAN / PIC_ERR_TIMEOUT).
+   error word (PIC_ERR_CAPACITY / PIC_ERR_CFL / PIC_ERR_NAN).
    Paper: one step of the particle-in-cell loop the paper's runs use (the
    electromagnetic PIC method named in section "Effect of the hyperbolic
    rotation in Minkowski space"), with the current filtered against short
@@ -626,15 +626,15 @@ pic_status pic_filter_current_noalloc(int dim, int nx, int ny, int nz, int bc_z,
 
 /* ------------------------------------------------------- bounded waits */
 
-/* The library's wait on an mbarrier never spins without limit: it gives up
-   after a time budget, and its caller reports PIC_ERR_TIMEOUT instead of
-   hanging (no kernel of the step waits on one at present).  This call checks
-   the wait on the device: one CTA waits on an mbarrier that expects one arrival, which the
-   kernel makes (arrive = 1: PIC_OK) or withholds (arrive = 0: nothing ever
-   completes the phase, the wait runs out after budget_ms and the call
-   returns PIC_ERR_TIMEOUT).  No fault is raised either way.  budget_ms in
+/* A check of a wait on an mbarrier that never spins without limit: it gives
+   up after a time budget instead of hanging.  No kernel of the library waits
+   on an mbarrier at present; the call is kept for callers that check their
+   device with it.  One CTA waits on an mbarrier that expects one arrival,
+   which the kernel makes (arrive = 1: PIC_OK) or withholds (arrive = 0:
+   nothing ever completes the phase, the wait runs out after budget_ms and the
+   call returns PIC_ERR_TIMEOUT).  No fault is raised either way.  budget_ms in
    (0, 10000], else PIC_ERR_ARG; PIC_ERR_CUDA if a CUDA call fails.  The
-   paper has no counterpart: this is a check of the library's own waits. */
+   paper has no counterpart. */
 pic_status pic_wait_check(int arrive, double budget_ms, void *stream);
 
 /* ------------------------------------------------------------------ misc */

@@ -275,7 +275,6 @@ static pic_status check_device_error(pic_ctx *c)
     if (h & ERR_NAN) return fail(c, PIC_ERR_NAN, "a non-finite particle momentum or position was produced");
     if (h & ERR_CFL) return fail(c, PIC_ERR_CFL, "a particle moved one cell or more in one step");
     if (h & ERR_CAPACITY) return fail(c, PIC_ERR_CAPACITY, "a tile bucket overflowed (raise slots_per_cell)");
-    if (h & ERR_TIMEOUT) return fail(c, PIC_ERR_TIMEOUT, "a bounded device wait ran out (a staged copy did not land)");
     return fail(c, PIC_ERR_STATE, "a particle was found outside its tile bucket");
 }
 

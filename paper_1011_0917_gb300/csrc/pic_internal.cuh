@@ -32,7 +32,7 @@
 
 namespace pic {
 
-enum : unsigned { ERR_CAPACITY = 1u, ERR_CFL = 2u, ERR_NAN = 4u, ERR_TILE = 8u, ERR_TIMEOUT = 16u };
+enum : unsigned { ERR_CAPACITY = 1u, ERR_CFL = 2u, ERR_NAN = 4u, ERR_TILE = 8u };
 
 // Bit 31 of an electron's cell word: the electron is paired with a drifting ion
 // at its own position that has moved exactly like it since both were placed
@@ -896,7 +896,6 @@ void launch_window_particles(const Geom &g, const Species<real> &in, const Speci
 template <typename real>
 void launch_yee(const Geom &g, real *const F[9], real *const F1[6], double dt, double hx, double hy, double hz,
                 cudaStream_t s);
-// (err: the device error word for a bounded wait that ran out; may be null)
 template <typename real>
 void launch_filter(const Geom &g, real *const J[3], real *tmp, int npass, cudaStream_t s);
 // all passes from src (3 contiguous components, left unchanged) into J;
