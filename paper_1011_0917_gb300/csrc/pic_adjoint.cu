@@ -1095,9 +1095,9 @@ void launch_adj_planes(const Geom &g, const real *F, int nc, unsigned char *near
     const int n = (g.nz + 1) * nc, cap = device_sms() * 32;
     if (g.plane <= kWarpPlane) {
         const int blocks = (n + 3) / 4;
-        launch_chained(chained(g), adj_planes_kernel<real, true>, (unsigned)(blocks < cap ? blocks : cap), 128, 0, s, g, F, nc, near);
+        launch_chained(adj_planes_kernel<real, true>, (unsigned)(blocks < cap ? blocks : cap), 128, 0, s, g, F, nc, near);
     } else {
-        launch_chained(chained(g), adj_planes_kernel<real, false>, (unsigned)(n < cap ? n : cap), 128, 0, s, g, F, nc, near);
+        launch_chained(adj_planes_kernel<real, false>, (unsigned)(n < cap ? n : cap), 128, 0, s, g, F, nc, near);
     }
 }
 
@@ -1107,11 +1107,11 @@ void launch_adj_planes(const Geom &g, const real *F, int nc, unsigned char *near
     if (a.n <= 0) return;                                                                       \
     const unsigned grid = adj_grid(a.n, 256);                                                   \
     if (a.g.dim == 3) {                                                                         \
-        if (a.g.shape == 1) launch_chained(chained(a.g), kernel<real, 3, 1>, grid, 256, 0, s, a);                         \
-        else launch_chained(chained(a.g), kernel<real, 3, 2>, grid, 256, 0, s, a);                                        \
+        if (a.g.shape == 1) launch_chained(kernel<real, 3, 1>, grid, 256, 0, s, a);                         \
+        else launch_chained(kernel<real, 3, 2>, grid, 256, 0, s, a);                                        \
     } else {                                                                                    \
-        if (a.g.shape == 1) launch_chained(chained(a.g), kernel<real, 2, 1>, grid, 256, 0, s, a);                         \
-        else launch_chained(chained(a.g), kernel<real, 2, 2>, grid, 256, 0, s, a);                                        \
+        if (a.g.shape == 1) launch_chained(kernel<real, 2, 1>, grid, 256, 0, s, a);                         \
+        else launch_chained(kernel<real, 2, 2>, grid, 256, 0, s, a);                                        \
     }
 
 template <typename real>
@@ -1137,16 +1137,16 @@ void launch_adj_yee(const Geom &g, real *lE[3], real *lB[3], real *lE0[3], real 
     const unsigned grid = adj_grid((int64_t)(g.nz + 1) * g.plane, 256);
     const real h = (real)(0.5 * dt);
     // B^{n+1} = B' - h curl E^{n+1}
-    launch_chained(chained(g), adj_curl_e_t_kernel<real>, grid, 256, 0, s, g, lE[0], lE[1], lE[2], lB[0], lB[1], lB[2], (real)(h / hz),
+    launch_chained(adj_curl_e_t_kernel<real>, grid, 256, 0, s, g, lE[0], lE[1], lE[2], lB[0], lB[1], lB[2], (real)(h / hz),
                                                   (real)(h / hx), (real)(h / hy), near, g.nz + 1);
     // E^{n+1} = E^n + dt (curl B' - 2 pi J), Mur on the z ends
-    launch_chained(chained(g), adj_e_update_t_kernel<real>, grid, 256, 0, s, g, lE[0], lE[1], lE[2], pE[0], pE[1], pE[2], lE0[0], lE0[1],
+    launch_chained(adj_e_update_t_kernel<real>, grid, 256, 0, s, g, lE[0], lE[1], lE[2], pE[0], pE[1], pE[2], lE0[0], lE0[1],
                                                     lE0[2], lJ[0], lJ[1], lJ[2], (real)((dt - hz) / (dt + hz)),
                                                     (real)(-kTwoPiD * dt));
-    launch_chained(chained(g), adj_curl_b_t_kernel<real>, grid, 256, 0, s, g, pE[0], pE[1], pE[2], lB[0], lB[1], lB[2], (real)(dt / hz),
+    launch_chained(adj_curl_b_t_kernel<real>, grid, 256, 0, s, g, pE[0], pE[1], pE[2], lB[0], lB[1], lB[2], (real)(dt / hz),
                                                   (real)(dt / hx), (real)(dt / hy));
     // B' = B^n - h curl E^n
-    launch_chained(chained(g), adj_curl_e_t_kernel<real>, grid, 256, 0, s, g, lE0[0], lE0[1], lE0[2], lB[0], lB[1], lB[2], (real)(h / hz),
+    launch_chained(adj_curl_e_t_kernel<real>, grid, 256, 0, s, g, lE0[0], lE0[1], lE0[2], lB[0], lB[1], lB[2], (real)(h / hz),
                                                   (real)(h / hx), (real)(h / hy), (unsigned char *)nullptr, 0);
 }
 
@@ -1154,7 +1154,7 @@ template <typename real>
 void launch_adj_antenna(const Geom &g, const real *lJ, int pol, int ka, double hx, double hy, double xc, double yc,
                         double waist, double fa, double fw, double *s, cudaStream_t st)
 {
-    launch_chained(chained(g), adj_antenna_kernel<real>, adj_grid(g.plane, 256), 256, 0, st, g, lJ, pol, ka, hx, hy, xc, yc,
+    launch_chained(adj_antenna_kernel<real>, adj_grid(g.plane, 256), 256, 0, st, g, lJ, pol, ka, hx, hy, xc, yc,
                                                                       1.0 / (waist * waist), fa, fw, s);
 }
 

@@ -729,7 +729,7 @@ void launch_yee(const Geom &g, real *const F[9], real *const F1[6], double dt, d
         a.nchunks = (nzo + a.cz - 1) / a.cz;
         const int64_t nitems = (int64_t)nstrip * a.nchunks, nblocks = (nitems + 7) / 8;
         if (record_launch(kBPYee, launch_yee2d_batch<real>, a, nblocks)) return;
-        launch_chained(chained(g), yee2d_kernel<real>, (unsigned)nblocks, 256, 0, s, a, nitems);
+        launch_chained(yee2d_kernel<real>, (unsigned)nblocks, 256, 0, s, a, nitems);
         return;
     }
     {
@@ -738,7 +738,7 @@ void launch_yee(const Geom &g, real *const F[9], real *const F1[6], double dt, d
         a.nchunks = (nzo + a.cz - 1) / a.cz;
         const int64_t nblocks = ncol * a.nchunks;
         if (record_launch(kBPYee, launch_yee3d_batch<real>, a, nblocks)) return;
-        launch_chained(chained(g), yee3d_kernel<real>, (unsigned)nblocks, 512, 0, s, a);
+        launch_chained(yee3d_kernel<real>, (unsigned)nblocks, 512, 0, s, a);
     }
 }
 
@@ -1166,7 +1166,7 @@ static void launch_march(const Geom &g, const real *in, real *out, cudaStream_t 
         if (record_launch(kBPFilter, launch_filter2d_batch<real, H>, MarchArgs<real>{g, in, out, cz, nchunks},
                           nblocks))
             return;
-        launch_chained(chained(g), filter2d_kernel<real, H>, (unsigned)nblocks, 256, 0, s, g, in, out, cz, nchunks);
+        launch_chained(filter2d_kernel<real, H>, (unsigned)nblocks, 256, 0, s, g, in, out, cz, nchunks);
     } else {
         constexpr int OWN = 32 - 2 * H;
         const int64_t ncol = (int64_t)((g.nx + OWN - 1) / OWN) * ((g.ny + OWN - 1) / OWN);
@@ -1177,7 +1177,7 @@ static void launch_march(const Geom &g, const real *in, real *out, cudaStream_t 
         if (record_launch(kBPFilter, launch_filter3d_batch<real, H>, MarchArgs<real>{g, in, out, cz, nchunks},
                           nblocks))
             return;
-        launch_chained(chained(g), filter3d_kernel<real, H>, (unsigned)nblocks, 512, 0, s, g, in, out, cz, nchunks);
+        launch_chained(filter3d_kernel<real, H>, (unsigned)nblocks, 512, 0, s, g, in, out, cz, nchunks);
     }
 }
 
@@ -1306,7 +1306,7 @@ void launch_antenna(const Geom &g, real *J, int pol, int ka, double j0, double h
     const AntennaArgs<real> a{g, J, pol, ka, j0, hx, hy, xc, yc, 1.0 / (waist * waist), j0p};
     const unsigned nb = grid_for(g.plane, 256);
     if (record_launch(kBPAntenna, launch_antenna_batch<real>, a, (int64_t)nb)) return;
-    launch_chained(chained(g), antenna_kernel<real>, (unsigned)nb, 256, 0, s, a);
+    launch_chained(antenna_kernel<real>, (unsigned)nb, 256, 0, s, a);
 }
 
 // ---------------------------------------------------------------- zeroing
@@ -1343,18 +1343,24 @@ __global__ void __launch_bounds__(256) zero_kernel(real *p, int64_t n, unsigned 
     for (int64_t o = first; o < m; o += stride) q[o] = 0;
 }
 
+// Values that zero_kernel takes, at most.  On small arrays it saves the gap
+// that a memset makes between two kernels (3D 16 x 16 x 32 cells 65 -> 62 us a
+// step); on large ones the two are alike (12.6M values 1056 us a step with the
+// kernel, 1059 with the memset; 100M values 6827 and 6826).
+constexpr int64_t kZeroKernelMax = 9 << 20;
+
 // returns the kernels it launches
 template <typename real>
 static int zero_launch(real *p, int64_t n, unsigned char *q, int64_t m, cudaStream_t s)
 {
     // a large array, or one off the 16-byte grid (J of an odd grid, zeroed
     // by itself): a plain memset
-    if (n > 3 * kChainNodes || reinterpret_cast<uintptr_t>(p) % 16 != 0) {
+    if (n > kZeroKernelMax || reinterpret_cast<uintptr_t>(p) % 16 != 0) {
         cudaMemsetAsync(p, 0, (size_t)n * sizeof(real), s);
         n = 0;
         if (m == 0) return 0;
     }
-    launch_chained(true, zero_kernel<real>, grid_for(n / 4 + 1, 256), 256, 0, s, p, n, q, m);
+    launch_chained(zero_kernel<real>, grid_for(n / 4 + 1, 256), 256, 0, s, p, n, q, m);
     return 1;
 }
 

@@ -259,7 +259,7 @@ void launch_inject(const InjectArgs &a, cudaStream_t s)
     if (record_launch(kBPInject, a.precision == 0 ? launch_inject_batch<float> : launch_inject_batch<double>, a,
                       blocks))
         return;
-    launch_chained(chained(a.g), a.precision == 0 ? inject_kernel<float> : inject_kernel<double>, (unsigned)blocks,
+    launch_chained(a.precision == 0 ? inject_kernel<float> : inject_kernel<double>, (unsigned)blocks,
                    kInjectThreads, 0, s, a);
 }
 

@@ -757,27 +757,27 @@ extern thread_local bool g_capture;
 #ifdef __CUDACC__
 // Launches that follow one another on a stream.  A step on a small grid is a
 // chain of kernels of a few microseconds, and between two of them the GPU
-// stood still for one to two.  A kernel launched by launch_chained may be set
-// up while the one before it still runs: it starts with chain_begin(), which
-// lets its own successor be set up in turn and then waits until the kernel
-// before it has completed and its writes are visible.  Every such kernel
-// calls it first, in every thread, so a kernel that completes implies that all
-// before it did, and what the stream holds afterwards (copies, events, other
-// kernels) is ordered as ever.  Graph captures take plain launches, and so do
-// grids of more than kChainNodes nodes: 64 x 512 cells gained 3% of a step's
-// time, a 2D gradient on 128 x 1536 26%, 256 x 8192 cells 4%, but 128 x 128 x
-// 256 lost 2% and 256 x 256 x 512 3% (the waiting CTAs hold their places while
-// long kernels end).
-constexpr int64_t kChainNodes = 3 << 20;
-inline bool chained(const Geom &g) { return g.ncomp <= kChainNodes; }
-__device__ __forceinline__ void chain_begin()
-{
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
+// stood still for one to two.  A kernel launched by launch_chained may start
+// as soon as every CTA of the one before it has left (a plain launch waits
+// until that kernel's memory is flushed and it is retired as well); it begins
+// with chain_begin(), which waits until the kernel before has completed and
+// its writes are visible.  Every such kernel calls it first, in every thread,
+// so a kernel that completes implies that all before it did, and what the
+// stream holds afterwards (copies, events, other kernels) is ordered as ever.
+// A batch's graph captures take plain launches.
+//
+// The next kernel is not let in earlier (griddepcontrol.launch_dependents):
+// its CTAs then settle, waiting, on the first SMs that come free, and it runs
+// with most of them on a few SMs.  us a step, plain launches / let in at the
+// start of the kernel before / not let in early: 3D 48 x 48 x 64 cells 112 /
+// 154 / 99, 128 x 128 x 256 1073 / 1083 / 1059, 256 x 256 x 512 6847 / 6953 /
+// 6826; 2D 64 x 256 39.8 / 32.4 / 28.9, in FP64 125 / 146 / 115, 160 x 512
+// quadratic 59 / 77 / 48, 256 x 8192 198 / 187 / 183, 1024 x 8192 652 / 644 /
+// 638.
+__device__ __forceinline__ void chain_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // (cluster: CTAs per thread-block cluster)
 template <typename... P, typename... A>
-inline void launch_clusters(bool chain, unsigned cluster, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem,
+inline void launch_clusters(unsigned cluster, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem,
                             cudaStream_t s, A... args)
 {
     cudaLaunchConfig_t c{};
@@ -787,7 +787,7 @@ inline void launch_clusters(bool chain, unsigned cluster, void (*kernel)(P...), 
     c.stream = s;
     cudaLaunchAttribute at[2] = {};
     c.attrs = at;
-    if (chain && !g_capture) {
+    if (!g_capture) {
         at[c.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         at[c.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
     }
@@ -800,10 +800,9 @@ inline void launch_clusters(bool chain, unsigned cluster, void (*kernel)(P...), 
     (void)cudaLaunchKernelEx(&c, kernel, P(args)...);
 }
 template <typename... P, typename... A>
-inline void launch_chained(bool chain, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
-                           A... args)
+inline void launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args)
 {
-    launch_clusters(chain, 1, kernel, grid, block, smem, s, args...);
+    launch_clusters(1, kernel, grid, block, smem, s, args...);
 }
 
 // the run owning work item `item`: the last r with start[r] <= item

@@ -59,12 +59,12 @@ static void launch_push_z(const PushArgs<real> &a, bool ions, cudaStream_t s)
         if (!ions && (a.g.ntiles < sms || a.g.ntiles * kSplit <= sms * MinBlocks<real, DIM>::value)) {
             auto ks = push_split_kernel<real, DIM, S, TX, TY, TZ, REL>;
             if (smem > 48 * 1024) cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            launch_clusters(chained(a.g), kSplit, ks, (unsigned)(a.g.ntiles * kSplit), BlockOf<real, DIM>::value, smem, s, a);
+            launch_clusters(kSplit, ks, (unsigned)(a.g.ntiles * kSplit), BlockOf<real, DIM>::value, smem, s, a);
             return;
         }
     }
     const int64_t grid = a.g.ntiles < 2147483647LL ? a.g.ntiles : 2147483647LL;
-    launch_chained(chained(a.g), k, (unsigned)grid, BlockOf<real, DIM>::value, smem, s, a);
+    launch_chained(k, (unsigned)grid, BlockOf<real, DIM>::value, smem, s, a);
 }
 
 // records in relative form (and their ions) take the REL kernels
