@@ -343,21 +343,35 @@ __global__ void __launch_bounds__(256) sort_cells_kernel(SortArgs<real> a)
         for (int p = tid; p < n; p += blockDim.x) {
             const int64_t s0 = bucket_slot(t, g.cap, n_lo, n_hi, p), s = a.in.r(s0);
             const int64_t d0 = t * (int64_t)g.cap + (sorted ? atomicAdd(&cnt[key[p]], 1) : p), d = a.out.r(d0);
-            a.out.ox[d] = a.in.ox[s];
-            if (a.in.oy) a.out.oy[d] = a.in.oy[s];
-            a.out.oz[d] = a.in.oz[s];
-            a.out.w[d] = a.in.w[s];
+            // (all of a record's loads before its stores, which might alias them)
+            const real ox = a.in.ox[s], oy = a.in.oy ? a.in.oy[s] : real(0), oz = a.in.oz[s], w = a.in.w[s];
+            real ux = 0, uy = 0, uz = 0, dlx = 0, dly = 0, dlz = 0;
+            const int32_t cell = a.in.cell[a.in.c(s0)];
             if (a.in.ux) {
-                a.out.ux[d] = a.in.ux[s];
-                a.out.uy[d] = a.in.uy[s];
-                a.out.uz[d] = a.in.uz[s];
+                ux = a.in.ux[s];
+                uy = a.in.uy[s];
+                uz = a.in.uz[s];
             }
             if (a.in.dlx) {
-                a.out.dlx[d] = a.in.dlx[s];
-                if (a.in.dly) a.out.dly[d] = a.in.dly[s];
-                a.out.dlz[d] = a.in.dlz[s];
+                dlx = a.in.dlx[s];
+                dly = a.in.dly ? a.in.dly[s] : real(0);
+                dlz = a.in.dlz[s];
             }
-            a.out.cell[a.out.c(d0)] = a.in.cell[a.in.c(s0)];
+            a.out.ox[d] = ox;
+            if (a.in.oy) a.out.oy[d] = oy;
+            a.out.oz[d] = oz;
+            a.out.w[d] = w;
+            if (a.in.ux) {
+                a.out.ux[d] = ux;
+                a.out.uy[d] = uy;
+                a.out.uz[d] = uz;
+            }
+            if (a.in.dlx) {
+                a.out.dlx[d] = dlx;
+                if (a.in.dly) a.out.dly[d] = dly;
+                a.out.dlz[d] = dlz;
+            }
+            a.out.cell[a.out.c(d0)] = cell;
             if (a.in.id) a.out.id[d0] = a.in.id[s0];
         }
         if (tid == 0) {
