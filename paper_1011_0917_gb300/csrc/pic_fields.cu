@@ -822,7 +822,9 @@ struct MarchArgs {
 // All H passes (H <= 4) along all axes in one march up z with the planes in
 // registers.  A pass (1/4, 1/2, 1/4) is a sum with the neighbour on one side
 // and then on the other, (v_i + v_i-1) + (v_i+1 + v_i): two adds, and one
-// exact scaling by a power of two ends all of them.  Along x the neighbours
+// exact scaling by a power of two ends all of them (until then the sums grow
+// by 2^(2H) per axis: FP32 currents beyond 2^(128 - 6H), 2e31 in 3D with four
+// passes, leave the range).  Along x the neighbours
 // are the lanes next door (shuffles: lane l holds column x0 + l - H, wrapped;
 // lanes H .. 31 - H own theirs).  Along z a pass keeps two registers of the
 // planes below and gives its result one plane late; with absorbing z a
@@ -835,8 +837,8 @@ struct MarchArgs {
 // pass's three planes and tested every node.  3D, against planes staged by TMA
 // in a ring of shared buffers with a stencil of width 2H + 1 per axis: 75 x 52
 // x 99 (H = 1) 24.5 -> 6.9 us, 128 x 128 x 256 (H = 2) 77 -> 40 us, 256 x 256 x
-// 512 349 -> 324 us (bound by issue slots: 3.3 TB/s of its 24 bytes a node would
-// take 120 us).
+// 512 349 -> 268 us (bound by issue slots: 3.0 TB/s of its 24 bytes a node,
+// which at the copy rate take 120 us).
 
 // one chunk of planes of the march: walks k from z0 - H to z1 - 1 + H
 template <typename real>
@@ -970,36 +972,53 @@ __device__ __forceinline__ void filter2d_body(const Geom &g, const real *in, rea
     else filter2d_march<real, H, false>(g, in, out, strip, z0, z1);
 }
 
-// In 3D a CTA of 16 warps holds 32 rows of 32 columns, two rows a warp: the x
-// passes are done for every row and the rows pass through shared memory (one
-// barrier per plane, two buffers in turn; FP64: one buffer and two barriers),
-// where a warp takes the H rows on
-// either side of its own two for the y passes.  (32 - 2H)^2 of the 32^2
-// columns are the CTA's own.
-template <typename real> constexpr int kFilterBufs = sizeof(real) == 4 ? 2 : 1;
+// In 3D a CTA holds rows of 32 columns, two rows a warp: the x passes are done
+// for every row and the rows pass through shared memory (one barrier per
+// plane, two buffers in turn), where a warp takes the H rows on either side of
+// its own two for the y passes.  Only columns H .. 31 - H and rows H .. rows -
+// 1 - H are the CTA's own (FP32, H = 2: 28^2 of 32^2).  Where the adds bound
+// it (FP64, and FP32 with H = 4; kFilterLean) the y passes of a row are the
+// binomial stencil of 2H + 1 rows, 2H adds and fused multiply-adds where
+// passes as sums take 2H^2 + 3H for two rows, and warps without an own row in
+// the grid leave out the y and z passes.  (In FP32 with H <= 3 the tests cost
+// more than they save: 200^3 cells, H = 2 116 us without, 123 with.)  FP64
+// takes 8 warps (16 rows): its pipe is full with one CTA per SM, and a grid of
+// 40^3 cells is 4 columns of 32 rows but 8 to 20 of 16.  FP64, us, sums over
+// 32 rows / this: 40^3 cells H = 1 66 / 40, H = 4 436 / 115; 100^3 H = 2 250 /
+// 176; 200^3 H = 4 5177 / 3306, H = 1 550 / 559.  FP32, H = 4: 200^3 239 / 213.
+template <typename real> constexpr int kFilterWarps = sizeof(real) == 4 ? 16 : 8;
+// resident CTAs per SM that the kernels are compiled for
+template <typename real, int H> constexpr int kFilterBlocks = H <= 2 ? 2 : 1;
+template <typename real, int H> constexpr bool kFilterLean = sizeof(real) == 8 || H == 4;
+// the binomial coefficient C(2H, i)
+template <int H> __device__ __forceinline__ constexpr int binomial(int i)
+{
+    int c = 1;
+    for (int q = 0; q < i; ++q) c = c * (2 * H - q) / (q + 1);
+    return c;
+}
 template <typename real, int H, bool INNER>
 __device__ __forceinline__ void filter3d_march(const Geom &g, const real *in, real *out, real *xs, const int sx,
                                                const int sy, const int z0, const int z1)
 {
     // rows of a component in shared memory: H more on either side of the
-    // CTA's 32, zero (they reach only rows the CTA does not own)
-    constexpr int OWN = 32 - 2 * H, CS = (32 + 2 * H) * 32;
-    for (int q = (int)threadIdx.x; q < kFilterBufs<real> * 3 * 2 * H * 32; q += 512) {
-        const int c = q / (2 * H * 32), e = q - c * (2 * H * 32);
-        xs[c * CS + e + (e >= H * 32 ? 32 * 32 : 0)] = real(0);
-    }
+    // CTA's, never written (only rows the CTA does not own would take them)
+    constexpr int ROWS = 2 * kFilterWarps<real>, OWNX = 32 - 2 * H, OWNY = ROWS - 2 * H, CS = (ROWS + 2 * H) * 32;
     const int lane = (int)(threadIdx.x & 31u), r0 = 2 * (int)(threadIdx.x >> 5);
-    const int x = sx * OWN + lane - H, y = sy * OWN + r0 - H;
+    const int x = sx * OWNX + lane - H, y = sy * OWNY + r0 - H;
     const int gx = x >= 0 && x < g.nx ? x : wrapi(x, g.nx);
     const bool ownx = lane >= H && lane < 32 - H && x < g.nx;
     int64_t col[2];
-    bool own[2];
+    bool own[2], row[2];
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
         const int yy = y + j, gy = yy >= 0 && yy < g.ny ? yy : wrapi(yy, g.ny);
         col[j] = (int64_t)gy * g.nx + gx;
-        own[j] = ownx && r0 + j >= H && r0 + j < 32 - H && yy < g.ny;
+        row[j] = r0 + j >= H && r0 + j < ROWS - H && yy < g.ny;
+        own[j] = ownx && row[j];
     }
+    // (uniform over the warp)
+    const bool used = !kFilterLean<real, H> || y < g.ny + H, mine = !kFilterLean<real, H> || row[0] || row[1];
     const real scale = real(1.0 / (double)(1 << (6 * H)));
     FilterWalk<real> w(g, z0 - H);
     const unsigned dp = (unsigned)(g.plane * sizeof(real));
@@ -1014,57 +1033,69 @@ __device__ __forceinline__ void filter3d_march(const Geom &g, const real *in, re
     for (int c = 0; c < 3; ++c)
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
-            cur[c][j] = ld(c, j, z0 - H);
+            cur[c][j] = used ? ld(c, j, z0 - H) : real(0);
 #pragma unroll
             for (int p = 0; p < H; ++p) pa[c][j][p] = pb[c][j][p] = real(0);
         }
-    real *mine = xs + (r0 + H) * 32 + lane;  // [buffer][component][row][lane]
+    real *at = xs + (r0 + H) * 32 + lane;  // [buffer][component][row][lane]
     // lane l < 12 prefetches a line of component l / 4's row r0 + (l / 2) % 2
     const int64_t ca = __shfl_sync(0xffffffffu, col[0], (lane & 1) ? 31 : 0),
                   cb = __shfl_sync(0xffffffffu, col[1], (lane & 1) ? 31 : 0);
     const real *pf = in + (lane >> 2) * g.ncomp + w.off + (kAhead + 1) * g.plane + ((lane & 2) ? cb : ca);
     int64_t o = (int64_t)(z0 - 2 * H) * g.plane;  // plane k - H
     for (int k = z0 - H; k < z1 + H; ++k) {
-        if (INNER && lane < 12 && k + kAhead + 1 < z1 + H) prefetch_l2(pf);
+        if (INNER && used && lane < 12 && k + kAhead + 1 < z1 + H) prefetch_l2(pf);
         pf += g.plane;
         const unsigned bo[2] = {b[0] - H * dp, b[1] - H * dp};  // plane k - H
         b[0] += dp;
         b[1] += dp;
         if (!INNER) w.next();
+        real *buf = at + (k & 1) * 3 * CS;
         real nxt[3][2];
+        if (used) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c)
+            for (int c = 0; c < 3; ++c)
 #pragma unroll
-            for (int j = 0; j < 2; ++j) nxt[c][j] = ld(c, j, k + 1);
-        real *buf = mine + (kFilterBufs<real> == 2 ? (k & 1) * 3 * CS : 0);
-        if (kFilterBufs<real> == 1) __syncthreads();
+                for (int j = 0; j < 2; ++j) nxt[c][j] = ld(c, j, k + 1);
 #pragma unroll
-        for (int c = 0; c < 3; ++c)
+            for (int c = 0; c < 3; ++c)
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                cur[c][j] = filter_x<real, H>(cur[c][j]);
-                buf[c * CS + j * 32] = cur[c][j];
-            }
+                for (int j = 0; j < 2; ++j) {
+                    cur[c][j] = filter_x<real, H>(cur[c][j]);
+                    buf[c * CS + j * 32] = cur[c][j];
+                }
+        }
         __syncthreads();
-        const bool w0 = own[0] && k >= z0 + H, w1 = own[1] && k >= z0 + H;
+        if (mine) {
+            const bool w0 = own[0] && k >= z0 + H, w1 = own[1] && k >= z0 + H;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            real v[2 * H + 2];  // rows r0 - H .. r0 + 1 + H
+            for (int c = 0; c < 3; ++c) {
+                real v[2 * H + 2];  // rows r0 - H .. r0 + 1 + H
 #pragma unroll
-            for (int q = 0; q < 2 * H + 2; ++q) {
-                const int d = q - H;
-                v[q] = d == 0 || d == 1 ? cur[c][d & 1] : buf[c * CS + d * 32];
-            }
+                for (int q = 0; q < 2 * H + 2; ++q) {
+                    const int d = q - H;
+                    v[q] = d == 0 || d == 1 ? cur[c][d & 1] : buf[c * CS + d * 32];
+                }
+                if (!kFilterLean<real, H>) {
 #pragma unroll
-            for (int p = 0; p < 2 * H; ++p)
+                    for (int p = 0; p < 2 * H; ++p)
 #pragma unroll
-                for (int q = 0; q < 2 * H + 1 - p; ++q) v[q] = v[q] + v[q + 1];
+                        for (int q = 0; q < 2 * H + 1 - p; ++q) v[q] = v[q] + v[q + 1];
+                }
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const real t = filter_z<real, H, INNER>(v[j], pa[c][j], pb[c][j], w, c, k);
-                if (j == 0 ? w0 : w1) {
-                    if (INNER) elem(out + c * g.ncomp, bo[j]) = t * scale;
-                    else out[c * g.ncomp + o + col[j]] = k - H > (c == 2 ? w.zmax_z : w.zmax_xy) ? real(0) : t * scale;
+                for (int j = 0; j < 2; ++j) {
+                    real t = v[j];
+                    if (kFilterLean<real, H>) {
+                        t += v[j + 2 * H];
+#pragma unroll
+                        for (int q = 1; q < H; ++q) t += real(binomial<H>(q)) * (v[j + q] + v[j + 2 * H - q]);
+                        t += real(binomial<H>(H)) * v[j + H];
+                    }
+                    t = filter_z<real, H, INNER>(t, pa[c][j], pb[c][j], w, c, k);
+                    if (j == 0 ? w0 : w1) {
+                        if (INNER) elem(out + c * g.ncomp, bo[j]) = t * scale;
+                        else out[c * g.ncomp + o + col[j]] = k - H > (c == 2 ? w.zmax_z : w.zmax_xy) ? real(0) : t * scale;
+                    }
                 }
             }
         }
@@ -1080,18 +1111,17 @@ template <typename real, int H>
 __device__ __forceinline__ void filter3d_item(const Geom &g, const real *in, real *out, int cz, int nchunks,
                                               int64_t item)
 {
-    __shared__ real xs[kFilterBufs<real> * 3 * (32 + 2 * H) * 32];
-    constexpr int OWN = 32 - 2 * H;
-    const int nsx = (g.nx + OWN - 1) / OWN, nsy = (g.ny + OWN - 1) / OWN;
+    constexpr int ROWS = 2 * kFilterWarps<real>, OWNX = 32 - 2 * H, OWNY = ROWS - 2 * H;
+    __shared__ real xs[2 * 3 * (ROWS + 2 * H) * 32];
+    const int nsx = (g.nx + OWNX - 1) / OWNX, nsy = (g.ny + OWNY - 1) / OWNY;
     const int sx = (int)(item % nsx), sy = (int)((item / nsx) % nsy), ch = (int)(item / ((int64_t)nsx * nsy));
     const int z0 = ch * cz, z1 = ch == nchunks - 1 ? g.nz + 1 : z0 + cz;
     if (z0 >= H && z1 + H <= g.nz - 1 && small_offsets<real>(g)) filter3d_march<real, H, true>(g, in, out, xs, sx, sy, z0, z1);
     else filter3d_march<real, H, false>(g, in, out, xs, sx, sy, z0, z1);
 }
 
-// FP32: 64 registers a thread, two CTAs per SM
 template <typename real, int H>
-__global__ void __launch_bounds__(512, (sizeof(real) == 4 && H <= 2 ? 2 : 1))
+__global__ void __launch_bounds__((32 * kFilterWarps<real>), (kFilterBlocks<real, H>))
     filter3d_kernel(Geom g, const real *in, real *out, int cz, int nchunks)
 {
     chain_begin();
@@ -1099,7 +1129,7 @@ __global__ void __launch_bounds__(512, (sizeof(real) == 4 && H <= 2 ? 2 : 1))
 }
 
 template <typename real, int H>
-__global__ void __launch_bounds__(512, (sizeof(real) == 4 && H <= 2 ? 2 : 1))
+__global__ void __launch_bounds__((32 * kFilterWarps<real>), (kFilterBlocks<real, H>))
     filter3d_batch_kernel(const MarchArgs<real> *__restrict__ runs, const int64_t *__restrict__ start, int n)
 {
     __shared__ __align__(16) MarchArgs<real> sa;
@@ -1112,10 +1142,15 @@ static void launch_filter3d_batch(const void *args, const int64_t *start, int n,
                                   cudaStream_t s)
 {
     filter3d_batch_kernel<real, H>
-        <<<(unsigned)total, 512, 0, s>>>(static_cast<const MarchArgs<real> *>(args), start, n);
+        <<<(unsigned)total, 32 * kFilterWarps<real>, 0, s>>>(static_cast<const MarchArgs<real> *>(args), start, n);
 }
 
-// one warp per (strip, chunk) item
+// one warp per (strip, chunk) item; in FP64 two warps a CTA, so that few items
+// share no SM's FP64 pipe while others idle
+template <typename real> constexpr int kFilter2Warps = sizeof(real) == 4 ? 8 : 2;
+// (FP64) warps that fill an SM's FP64 pipe; us, 4 / 8: 1000 x 1000 cells (H =
+// 1) 78 / 62, 256 x 8192 (H = 4) 374 / 549, else within 15%
+template <int H> constexpr int kFilter2Resident = H <= 3 ? 8 : 4;
 template <typename real, int H>
 __device__ __forceinline__ void filter2d_items(const Geom &g, const real *in, real *out, int cz, int nchunks,
                                                int64_t item)
@@ -1126,19 +1161,20 @@ __device__ __forceinline__ void filter2d_items(const Geom &g, const real *in, re
 }
 
 template <typename real, int H>
-__global__ void __launch_bounds__(256) filter2d_kernel(Geom g, const real *in, real *out, int cz, int nchunks)
+__global__ void __launch_bounds__((32 * kFilter2Warps<real>))
+    filter2d_kernel(Geom g, const real *in, real *out, int cz, int nchunks)
 {
     chain_begin();
-    filter2d_items<real, H>(g, in, out, cz, nchunks, (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5));
+    filter2d_items<real, H>(g, in, out, cz, nchunks, (int64_t)blockIdx.x * kFilter2Warps<real> + (threadIdx.x >> 5));
 }
 
 template <typename real, int H>
-__global__ void __launch_bounds__(256) filter2d_batch_kernel(const MarchArgs<real> *__restrict__ runs,
-                                                             const int64_t *__restrict__ start, int n)
+__global__ void __launch_bounds__((32 * kFilter2Warps<real>))
+    filter2d_batch_kernel(const MarchArgs<real> *__restrict__ runs, const int64_t *__restrict__ start, int n)
 {
     __shared__ __align__(16) MarchArgs<real> sa;
     const int64_t b = batch_block(runs, start, n, &sa);
-    filter2d_items<real, H>(sa.g, sa.in, sa.out, sa.cz, sa.nchunks, b * 8 + (threadIdx.x >> 5));
+    filter2d_items<real, H>(sa.g, sa.in, sa.out, sa.cz, sa.nchunks, b * kFilter2Warps<real> + (threadIdx.x >> 5));
 }
 
 template <typename real, int H>
@@ -1146,7 +1182,7 @@ static void launch_filter2d_batch(const void *args, const int64_t *start, int n,
                                   cudaStream_t s)
 {
     filter2d_batch_kernel<real, H>
-        <<<(unsigned)total, 256, 0, s>>>(static_cast<const MarchArgs<real> *>(args), start, n);
+        <<<(unsigned)total, 32 * kFilter2Warps<real>, 0, s>>>(static_cast<const MarchArgs<real> *>(args), start, n);
 }
 
 template <typename real, int DIM, int H>
@@ -1154,30 +1190,37 @@ static void launch_march(const Geom &g, const real *in, real *out, cudaStream_t 
 {
     const int nzo = g.nz + 1;
     if constexpr (DIM == 2) {
-        // the register march (2D grids): chunks of 4..64 planes, as many as
-        // leave about 24 warps per SM
-        constexpr int OWN = 32 - 2 * H;
+        // FP32: chunks of 4..64 planes, as many as leave about 24 warps per SM.
+        // FP64: the FP64 pipe of an SM is full with a few warps, beyond which
+        // shorter chunks only repeat their halos.
+        constexpr int OWN = 32 - 2 * H, NW = kFilter2Warps<real>;
         const int nstrip = (g.nx + OWN - 1) / OWN;
-        int64_t czl = (int64_t)nzo * nstrip * batch_runs() / ((int64_t)device_sms() * 24);
-        int cz = (int)(czl < 4 ? 4 : (czl > 64 ? 64 : czl));
+        int cz;
+        if (sizeof(real) == 4) {
+            const int64_t czl = (int64_t)nzo * nstrip * batch_runs() / ((int64_t)device_sms() * 24);
+            cz = (int)(czl < 4 ? 4 : (czl > 64 ? 64 : czl));
+        } else {
+            cz = chunk_planes(nzo, (int64_t)nstrip * batch_runs(), (int64_t)device_sms() * kFilter2Resident<H>, 2 * H, 4, 64);
+        }
         if (cz > nzo) cz = nzo;
         const int nchunks = (nzo + cz - 1) / cz;
-        const int64_t nblocks = ((int64_t)nstrip * nchunks + 7) / 8;
+        const int64_t nblocks = ((int64_t)nstrip * nchunks + NW - 1) / NW;
         if (record_launch(kBPFilter, launch_filter2d_batch<real, H>, MarchArgs<real>{g, in, out, cz, nchunks},
                           nblocks))
             return;
-        launch_chained(filter2d_kernel<real, H>, (unsigned)nblocks, 256, 0, s, g, in, out, cz, nchunks);
+        launch_chained(filter2d_kernel<real, H>, (unsigned)nblocks, 32 * NW, 0, s, g, in, out, cz, nchunks);
     } else {
-        constexpr int OWN = 32 - 2 * H;
-        const int64_t ncol = (int64_t)((g.nx + OWN - 1) / OWN) * ((g.ny + OWN - 1) / OWN);
-        const int cz = chunk_planes(nzo, ncol * batch_runs(), (int64_t)device_sms() * (sizeof(real) == 4 && H <= 2 ? 2 : 1),
-                                    2 * H, 4, kChunk3);
+        // (FP64: waves of one CTA per SM, whose FP64 pipe it fills)
+        constexpr int OWNX = 32 - 2 * H, OWNY = 2 * kFilterWarps<real> - 2 * H;
+        const int64_t ncol = (int64_t)((g.nx + OWNX - 1) / OWNX) * ((g.ny + OWNY - 1) / OWNY);
+        const int cz = chunk_planes(nzo, ncol * batch_runs(),
+                                    (int64_t)device_sms() * (sizeof(real) == 4 ? kFilterBlocks<real, H> : 1), 2 * H, 4, kChunk3);
         const int nchunks = (nzo + cz - 1) / cz;
         const int64_t nblocks = ncol * nchunks;
         if (record_launch(kBPFilter, launch_filter3d_batch<real, H>, MarchArgs<real>{g, in, out, cz, nchunks},
                           nblocks))
             return;
-        launch_chained(filter3d_kernel<real, H>, (unsigned)nblocks, 512, 0, s, g, in, out, cz, nchunks);
+        launch_chained(filter3d_kernel<real, H>, (unsigned)nblocks, 32 * kFilterWarps<real>, 0, s, g, in, out, cz, nchunks);
     }
 }
 
