@@ -95,7 +95,9 @@ struct Rec {
 // species' currents: ~1/(2 gamma^2) of the plasma's response in the lab, so
 // at gamma = 130 about 3e-8 of either species' current.  Each particle's
 // current must then be formed from a position exact far beyond FP32, and in
-// FP64 arithmetic, or the difference is rounding noise.  A record in relative
+// arithmetic far finer than FP32 (pairs of FP32 words in the FP32 build, see
+// ff; FP64 in the FP64 build), or the difference is rounding noise.  A record
+// in relative
 // form holds, per axis, a reference offset o in [0, 1) -- along z it moves
 // with exactly the arithmetic of a drifting ion, across it stays where the
 // particle was placed, i.e. it is its ion's path -- plus the departure dl
@@ -105,7 +107,7 @@ struct Rec {
 // for any record) and r the shift this function returns; its result is the
 // electron's offset in cell c, in [0, 1), for the gather.  The rounding of
 // o + dl here does not accumulate: it is redone from the exact pair every
-// step, and the current is deposited from the pair itself (in FP64).
+// step, and the current is deposited from the pair itself.
 template <typename real>
 __host__ __device__ inline real rel_actual(real o, real dl, int &r)
 {
@@ -401,9 +403,11 @@ __device__ __forceinline__ real drift_velocity(const Drift<real> &d, real dux, r
     return (duz * (real(2) + E) - d.U * p2) * (ig * d.ig * is);
 }
 
-// An unevaluated sum h + l of two FP32 values, |l| <= ulp(h) / 2: about 48
-// bits, from the error-free sum and product (Knuth, TAOCP 2, 4.2.2; Dekker,
-// Numer. Math. 18, 1971, with a fused multiply-add for the product's error).
+// An unevaluated sum h + l of two FP32 values, |l| <= ulp(h) / 2: 48 bits,
+// from the error-free sum and product (Knuth, TAOCP 2, 4.2.2; Dekker, Numer.
+// Math. 18, 1971, with a fused multiply-add for the product's error).  Sums and
+// products of pairs round their low words and drop a.l b.l: each is good to
+// about 46 bits of its larger operand.
 // FP64 arithmetic gives 2 lanes per SM and cycle here, FP32 128, of which one
 // of these operations takes 7 to 11.  The currents of records in relative
 // form use them: they need the records' exact positions and far more than
@@ -551,7 +555,7 @@ struct PushArgs {
     int fuse_ions;         // 1: the same CTA then moves and deposits the tile's ions
     IonSide<real> ions;    // (with fuse_ions) the ion sides and counters
     int rel;               // 1: electron records in relative form (rel_actual), currents
-                           //    of electrons and ions from FP64 arithmetic
+                           //    of electrons and ions in pairs of FP32 words (ff; FP64 build: FP64)
     unsigned *err;
 };
 
@@ -773,7 +777,11 @@ extern thread_local bool g_capture;
 // 154 / 99, 128 x 128 x 256 1073 / 1083 / 1059, 256 x 256 x 512 6847 / 6953 /
 // 6826; 2D 64 x 256 39.8 / 32.4 / 28.9, in FP64 125 / 146 / 115, 160 x 512
 // quadratic 59 / 77 / 48, 256 x 8192 198 / 187 / 183, 1024 x 8192 652 / 644 /
-// 638.
+// 638.  (In a process that has used more than about 8 streams every dependent
+// launch takes the GPU's front end longer.  There the early start would hide
+// more of it on 2D grids of some thousand tiles: 256 x 2048 80 / 66 / 69, 256 x
+// 4096 118 / 105 / 108, 256 x 8192 200 / 186 / 188; with one stream 79 / 68 /
+// 65, 118 / 110 / 103, 198 / 187 / 183.)
 __device__ __forceinline__ void chain_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // (cluster: CTAs per thread-block cluster)
 template <typename... P, typename... A>

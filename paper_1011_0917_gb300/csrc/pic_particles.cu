@@ -47,12 +47,16 @@ static void launch_push_z(const PushArgs<real> &a, bool ions, cudaStream_t s)
     auto k = ions ? ion_kernel<real, DIM, S, TX, TY, TZ, REL> : push_kernel<real, DIM, S, TX, TY, TZ, REL>;
     if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     // One CTA per tile, or kSplit (the default tile shapes) where the tiles are
-    // fewer than the SMs or kSplit CTAs for each are resident at once; beyond
-    // that the tiles fill the device and splitting them repeats their staging.
-    // us per pass, one CTA / kSplit: 64 x 512 cells (128 tiles, 16 steps) 784 /
-    // 581; FP64, 4 steps, 900 particles a tile: 64 tiles 1083 / 824, 96 tiles
-    // 1488 / 1067, 152 tiles 1069 / 1293; 3D: 125 tiles 416 / 395, 432 tiles
-    // 500 / 581; 2D: 304 tiles 693 / 705.
+    // fewer than the SMs or kSplit CTAs for each fit the CTAs per SM that the
+    // kernel is compiled for (in 3D FP64 shared memory holds one of the two);
+    // beyond that the tiles fill the device and splitting them repeats their
+    // staging.  us per step, one CTA / kSplit: 2D 64 tiles 34.0 / 28.9, 200
+    // tiles 34.3 / 31.5, 384 tiles 36.0 / 40.0; FP64 64 tiles 159 / 115; 3D 16
+    // tiles 72 / 48, 96 tiles 74 / 63.  us per pass of thermal plasmas: FP64, 900
+    // particles a tile, 96 tiles 1488 / 1067, 152 tiles 1069 / 1293; 3D 125 tiles
+    // 422 / 387, 432 tiles 500 / 581.  (Other tile shapes, which a caller asks
+    // for, are not compiled for it, to keep the kernels' number down: 32 x 8
+    // tiles of 64 x 512 cells would gain 8%, 8 x 8 x 4 tiles nothing.)
     constexpr bool kDefaultTile = DIM == 3 ? TZ == 8 : TX == 16;
     if constexpr (kDefaultTile) {
         const int64_t sms = device_sms();

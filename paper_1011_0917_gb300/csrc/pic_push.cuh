@@ -97,8 +97,8 @@ template <int SPLIT> __device__ __forceinline__ int stay_add(int *p, int n)
 // exact and associative, so a tile's sums do not depend on the order in which
 // its particles are processed, and they carry the contributions to 2^-K.
 // The "lo" word of a node sits LOFF words after its "hi" word.  FP64
-// accumulates in double.  Zero words (e.g. nodes of a window outside both
-// supports) are not added.
+// accumulates in double, and does not add zeros (e.g. nodes of a window
+// outside both supports); the FP32 words are added without a test.
 template <typename real> struct Acc { using type = double; };
 template <> struct Acc<float> { using type = int; };
 // bytes of a shared current tile of n values ("hi" and "lo" words in FP32), a multiple of 16
@@ -660,7 +660,9 @@ __device__ __forceinline__ int esirk_rel(double x0, double x1, double S0[S + 2],
 {
     return esirk_axis_g<S>(x0, x1, S0, DS, crossed);
 }
-// a position in the arithmetic of the deposit: r + (o + dl), exact
+// a position in the arithmetic of the deposit: r + (o + dl).  The pair of o and
+// dl is exact; adding the cell shift r (0 for most records) rounds its low word,
+// by at most 2^-48 of the position.
 template <typename T> __device__ __forceinline__ T rel_pos(int r, double o, double dl) { return (T)r + (o + dl); }
 template <typename T> __device__ __forceinline__ T rel_pos(int r, float o, float dl)
 {
