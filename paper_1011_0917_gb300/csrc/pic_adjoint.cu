@@ -390,7 +390,7 @@ template <typename real, int DIM, int S> struct AdjBlocks {
 template <typename real, int DIM, int S>
 __global__ void __launch_bounds__(256, (AdjBlocks<real, DIM, S>::push)) adj_push_kernel(AdjArgs<real> a)
 {
-    chain_begin();
+    chain_begin(a.g.early);
     constexpr int W = S + 2, WY = DIM == 3 ? W : 1;
     const Geom &g = a.g;
     const Drift<real> drift(a.u_drift, a.dtdh[2]);
@@ -562,7 +562,7 @@ __device__ __forceinline__ real adj_ion_vjp_one(const AdjArgs<real> &a, const Dr
 template <typename real, int DIM, int S>
 __global__ void __launch_bounds__(256, (AdjBlocks<real, DIM, S>::vjp)) adj_push_vjp_kernel(AdjArgs<real> a)
 {
-    chain_begin();
+    chain_begin(a.g.early);
     constexpr int W = S + 2, WY = DIM == 3 ? W : 1;
     const Geom &g = a.g;
     const Drift<real> drift(a.u_drift, a.dtdh[2]);
@@ -861,7 +861,7 @@ template <typename real>
 __global__ void adj_curl_e_t_kernel(Geom g, real *lEx, real *lEy, real *lEz, const real *lBx, const real *lBy,
                                     const real *lBz, real hz_, real hx_, real hy_, unsigned char *near, int nz1)
 {
-    chain_begin();
+    chain_begin(g.early);
     // (the masks the reverse step sets later start from zero)
     if (near)
         for (int k = (int)(blockIdx.x * blockDim.x + threadIdx.x); k < nz1; k += (int)(gridDim.x * blockDim.x)) near[k] = 0;
@@ -900,7 +900,7 @@ __global__ void adj_e_update_t_kernel(Geom g, const real *lE1x, const real *lE1y
                                       real *pEy, real *pEz, real *lE0x, real *lE0y, real *lE0z, real *lJx,
                                       real *lJy, real *lJz, real cm, real m2pidt)
 {
-    chain_begin();
+    chain_begin(g.early);
     const bool per = g.bc_z == 0;
     const int nk = g.nz + 1;
     const int64_t plane = g.plane;
@@ -943,7 +943,7 @@ template <typename real>
 __global__ void adj_curl_b_t_kernel(Geom g, const real *pEx, const real *pEy, const real *pEz, real *lBx,
                                     real *lBy, real *lBz, real dthz, real dthx, real dthy)
 {
-    chain_begin();
+    chain_begin(g.early);
     const bool per = g.bc_z == 0, d3 = g.dim == 3;
     const int nk = g.nz + 1;
     const int64_t plane = g.plane;
@@ -977,7 +977,7 @@ template <typename real>
 __global__ void adj_antenna_kernel(Geom g, const real *lJ, int pol, int ka, double hx, double hy, double xc,
                                    double yc, double inv_w2, double fa, double fw, double *s)
 {
-    chain_begin();
+    chain_begin(g.early);
     double s0 = 0, s1 = 0;
     for (int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; o < g.plane;
          o += (int64_t)gridDim.x * blockDim.x) {
@@ -1075,7 +1075,7 @@ __device__ __forceinline__ bool any_nonzero(const real *P, int n, int first, int
 template <typename real, bool WARP>
 __global__ void adj_planes_kernel(Geom g, const real *F, int nc, unsigned char *near)
 {
-    chain_begin();
+    chain_begin(g.early);
     const int nk = g.bc_z == 0 ? g.nz : g.nz + 1, n = nk * nc;
     const int per = WARP ? (int)(blockDim.x >> 5) : 1, mine = WARP ? (int)(threadIdx.x >> 5) : 0;
     const int first = WARP ? (int)(threadIdx.x & 31u) : (int)threadIdx.x, stride = WARP ? 32 : (int)blockDim.x;

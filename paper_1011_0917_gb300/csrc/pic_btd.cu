@@ -19,7 +19,7 @@ namespace pic {
 template <typename real>
 __global__ void btd_kernel(BtdArgs<real> a)
 {
-    chain_begin();
+    chain_begin(a.g.early);
     const int js = (int)blockIdx.y;
     const int idx = (int)(blockIdx.x * blockDim.x + threadIdx.x);
     const int kk = idx / a.nxs, is = idx - kk * a.nxs;

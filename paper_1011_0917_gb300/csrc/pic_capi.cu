@@ -656,17 +656,18 @@ static bool in_reach(const pic_ctx *c, const void *p)
     return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == c->device);
 }
 
-// bucket flat columns: from where they are when the context's device can read
-// them there, else through a copy in the staging (inactive) side
+// bucket flat columns: from where they are when the context's kernels can read
+// them there (in_place), else through a copy in the staging (inactive) side
 template <typename real>
-static pic_status upload_flat(pic_ctx *c, int sp, int64_t n, const void *const cols[kAttrs], int src_is_device)
+static pic_status upload_flat(pic_ctx *c, int sp, int64_t n, const void *const cols[kAttrs], int src_is_device,
+                              bool in_place)
 {
-    bool direct = src_is_device != 0;
+    bool direct = in_place;
     void *own[kAttrs] = {nullptr};
     for (int a = 0; a < kAttrs; ++a) {
         if (c->side[sp].off[a] == SIZE_MAX) continue;
         own[a] = const_cast<void *>(cols[a]);
-        direct = direct && cols[a] && (uintptr_t)cols[a] % attr_size(c, a) == 0 && in_reach(c, cols[a]);
+        direct = direct && cols[a] && (uintptr_t)cols[a] % attr_size(c, a) == 0;
     }
     if (direct) return bucket_flat<real>(c, sp, n, view_of<real>(own, 32, 32));
     void *dst[kAttrs];
@@ -717,7 +718,7 @@ static pic_status load_particles_t(pic_ctx *c, int sp, int64_t n, const double *
     const void *ptrs[kAttrs];
     for (int a = 0; a < kAttrs; ++a) ptrs[a] = cols[a].empty() ? nullptr : cols[a].data();
     c->wmax = std::max(c->wmax, wmax);
-    return upload_flat<real>(c, sp, n, ptrs, 0);
+    return upload_flat<real>(c, sp, n, ptrs, 0, false);
 }
 
 extern "C" pic_status pic_load_particles(pic_ctx *c, int sp, int64_t n, const double *state, const int64_t *ids)
@@ -2161,6 +2162,7 @@ static pic_status set_state_t(pic_ctx *c, const unsigned char *src, size_t src_b
     const size_t need = sizeof(StateHeader) + c->field_bytes + species_state_bytes(c, 0, h.n[0]) +
                         (c->ions_species ? species_state_bytes(c, 1, h.n[1]) : 0);
     if (src_bytes < need) return fail(c, PIC_ERR_ARG, "snapshot truncated");
+    const bool in_place = src_is_device && in_reach(c, src) && in_reach(c, src + need - 1);
     size_t o = sizeof(StateHeader);
     c->fset = 0;
     CUDA_TRY(c, cudaMemcpyAsync(c->fields, src + o, c->field_bytes, kind_in(src_is_device), c->stream));
@@ -2174,7 +2176,7 @@ static pic_status set_state_t(pic_ctx *c, const unsigned char *src, size_t src_b
             o += (size_t)h.n[sp] * attr_size(c, a);
         }
         if (h.n[sp] == 0) continue;
-        pic_status s = upload_flat<real>(c, sp, h.n[sp], cols, src_is_device);
+        pic_status s = upload_flat<real>(c, sp, h.n[sp], cols, src_is_device, in_place);
         if (s != PIC_OK) return s;
     }
     c->wmax = h.wmax;
@@ -2456,6 +2458,14 @@ static void adj_inject_out(pic_ctx *c, const AdjLayout &L, unsigned char *st, In
     ia.f_zeta = (double *)(B + L.zeta);
 }
 
+// while it lives, the kernels launched on this grid let their successors in
+// early (a gradient's, see launch_chained)
+struct EarlyLaunches {
+    Geom &g;
+    explicit EarlyLaunches(Geom &grid) : g(grid) { g.early = g.dim == 2 && g.ncomp >= kEarlyNodes; }
+    ~EarlyLaunches() { g.early = 0; }
+};
+
 // one flat step n: state/fields slot a -> slot b
 template <typename real>
 static void adj_step(pic_ctx *c, const AdjLayout &L, unsigned char *sa, unsigned char *sb, unsigned char *fa,
@@ -2465,7 +2475,7 @@ static void adj_step(pic_ctx *c, const AdjLayout &L, unsigned char *sa, unsigned
     const int64_t nc = c->g.ncomp;
     // the raw current goes to the filter's input buffer; the filter writes J
     real *J = (real *)(B + L.J), *R = (real *)(B + L.tmp);
-    launch_zero2<real>(R, 3 * nc, sa + L.fm, c->g.nz + 1, c->stream);
+    launch_zero2<real>(R, 3 * nc, sa + L.fm, c->g.nz + 1, c->g.early, c->stream);
     AdjArgs<real> a{};
     a.g = c->g;
     for (int q = 0; q < 3; ++q) {
@@ -2520,6 +2530,7 @@ template <typename real>
 static pic_status adj_forward_t(pic_ctx *c, const pic_adjoint_params *p, void *fields_out, bool defer)
 {
     auto &A = c->adj;
+    const EarlyLaunches early(c->g);
     const AdjLayout L =
         adj_layout(A.P, p->nsteps, p->checkpoint_every, p->sub_checkpoint_every, sizeof(real), c->g.ncomp,
                    c->g.dim == 3, c->g.nz + 1);
@@ -2612,6 +2623,7 @@ template <typename real>
 static pic_status adj_backward_t(pic_ctx *c, const void *cot)
 {
     auto &A = c->adj;
+    const EarlyLaunches early(c->g);
     const AdjLayout L = adj_layout(A.P, A.N, A.K, A.K2, sizeof(real), c->g.ncomp, c->g.dim == 3, c->g.nz + 1);
     unsigned char *B = A.buf;
     const int64_t nc = c->g.ncomp;

@@ -643,7 +643,7 @@ __device__ __forceinline__ void yee3d_item(const YeeArgs<real> &a, int64_t item)
 template <typename real>
 __global__ void __launch_bounds__(512, 2) yee3d_kernel(YeeArgs<real> a)
 {
-    chain_begin();
+    chain_begin(a.g.early);
     yee3d_item(a, (int64_t)blockIdx.x);
 }
 
@@ -677,7 +677,7 @@ __device__ __forceinline__ void yee2d_items(const YeeArgs<real> &a, int64_t item
 template <typename real>
 __global__ void __launch_bounds__(256) yee2d_kernel(YeeArgs<real> a, int64_t nitems)
 {
-    chain_begin();
+    chain_begin(a.g.early);
     yee2d_items(a, (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5), nitems);
 }
 
@@ -1124,7 +1124,7 @@ template <typename real, int H>
 __global__ void __launch_bounds__((32 * kFilterWarps<real>), (kFilterBlocks<real, H>))
     filter3d_kernel(Geom g, const real *in, real *out, int cz, int nchunks)
 {
-    chain_begin();
+    chain_begin(g.early);
     filter3d_item<real, H>(g, in, out, cz, nchunks, (int64_t)blockIdx.x);
 }
 
@@ -1164,7 +1164,7 @@ template <typename real, int H>
 __global__ void __launch_bounds__((32 * kFilter2Warps<real>))
     filter2d_kernel(Geom g, const real *in, real *out, int cz, int nchunks)
 {
-    chain_begin();
+    chain_begin(g.early);
     filter2d_items<real, H>(g, in, out, cz, nchunks, (int64_t)blockIdx.x * kFilter2Warps<real> + (threadIdx.x >> 5));
 }
 
@@ -1321,7 +1321,7 @@ __device__ __forceinline__ void antenna_body(const AntennaArgs<real> &a, int64_t
 template <typename real>
 __global__ void antenna_kernel(AntennaArgs<real> a)
 {
-    chain_begin();
+    chain_begin(a.g.early);
     antenna_body(a, (int64_t)blockIdx.x, (int64_t)gridDim.x);
 }
 
@@ -1376,9 +1376,9 @@ static void launch_zero_batch(const void *args, const int64_t *start, int n, int
 
 // n values at p (16-byte aligned) and m bytes at q
 template <typename real>
-__global__ void __launch_bounds__(256) zero_kernel(real *p, int64_t n, unsigned char *q, int64_t m)
+__global__ void __launch_bounds__(256) zero_kernel(real *p, int64_t n, unsigned char *q, int64_t m, int early)
 {
-    chain_begin();
+    chain_begin(early);
     const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
     constexpr int V = 16 / (int)sizeof(real);
     for (int64_t o = first; o < n / V; o += stride) reinterpret_cast<int4 *>(p)[o] = make_int4(0, 0, 0, 0);
@@ -1394,7 +1394,7 @@ constexpr int64_t kZeroKernelMax = 9 << 20;
 
 // returns the kernels it launches
 template <typename real>
-static int zero_launch(real *p, int64_t n, unsigned char *q, int64_t m, cudaStream_t s)
+static int zero_launch(real *p, int64_t n, unsigned char *q, int64_t m, int early, cudaStream_t s)
 {
     // a large array, or one off the 16-byte grid (J of an odd grid, zeroed
     // by itself): a plain memset
@@ -1403,7 +1403,7 @@ static int zero_launch(real *p, int64_t n, unsigned char *q, int64_t m, cudaStre
         n = 0;
         if (m == 0) return 0;
     }
-    launch_chained(zero_kernel<real>, grid_for(n / 4 + 1, 256), 256, 0, s, p, n, q, m);
+    launch_chained(zero_kernel<real>, grid_for(n / 4 + 1, 256), 256, 0, s, p, n, q, m, early);
     return 1;
 }
 
@@ -1413,13 +1413,13 @@ int launch_zero(real *p, int64_t n, cudaStream_t s)
     if (n <= 0) return 0;
     if (record_launch(kBPZero, launch_zero_batch<real>, ZeroArgs<real>{p, n}, (n + kZeroChunk - 1) / kZeroChunk))
         return 1;
-    return zero_launch(p, n, nullptr, 0, s);
+    return zero_launch(p, n, nullptr, 0, 0, s);
 }
 
 template <typename real>
-void launch_zero2(real *p, int64_t n, unsigned char *q, int64_t m, cudaStream_t s)
+void launch_zero2(real *p, int64_t n, unsigned char *q, int64_t m, int early, cudaStream_t s)
 {
-    zero_launch(p, n, q, m, s);
+    zero_launch(p, n, q, m, early, s);
 }
 
 // ------------------------------------------------------------ field sums
@@ -1490,7 +1490,7 @@ int launch_field_sums(const Geom &g, real *const F[9], double *partials, int max
                                        double, double, cudaStream_t, const double *);                   \
     template int launch_field_sums<real>(const Geom &, real *const[9], double *, int, cudaStream_t); \
     template int launch_zero<real>(real *, int64_t, cudaStream_t);                                      \
-    template void launch_zero2<real>(real *, int64_t, unsigned char *, int64_t, cudaStream_t);
+    template void launch_zero2<real>(real *, int64_t, unsigned char *, int64_t, int, cudaStream_t);
 PIC_FIELDS_INSTANTIATE(float)
 PIC_FIELDS_INSTANTIATE(double)
 

@@ -225,7 +225,7 @@ __device__ __forceinline__ void inject_body(const InjectArgs &a, const int64_t b
 template <typename real>
 __global__ void inject_kernel(InjectArgs a)
 {
-    chain_begin();
+    chain_begin(a.g.early);
     inject_body<real>(a, (int64_t)blockIdx.x, (int64_t)gridDim.x);
 }
 

@@ -50,6 +50,7 @@ struct Geom {
     int lt[3];          // log2 of the tile shape
     int nt[3];          // tiles per axis
     int cap;            // slots per tile
+    int early;          // its kernels let the next one on the stream in early (see launch_chained)
     int64_t plane;      // nx * ny
     int64_t ncomp;      // (nz + 1) * plane, elements per field component
     int64_t ntiles;
@@ -97,17 +98,16 @@ struct Rec {
 // current must then be formed from a position exact far beyond FP32, and in
 // arithmetic far finer than FP32 (pairs of FP32 words in the FP32 build, see
 // ff; FP64 in the FP64 build), or the difference is rounding noise.  A record
-// in relative
-// form holds, per axis, a reference offset o in [0, 1) -- along z it moves
-// with exactly the arithmetic of a drifting ion, across it stays where the
-// particle was placed, i.e. it is its ion's path -- plus the departure dl
-// from it, |dl| <= 1/2 (whole cells move between dl and the reference cell,
-// which is exact).  The position is c_ref + o + dl with c_ref = c + r, c the
-// stored cell (the one the electron is in, so that tiles and stencils are as
-// for any record) and r the shift this function returns; its result is the
-// electron's offset in cell c, in [0, 1), for the gather.  The rounding of
-// o + dl here does not accumulate: it is redone from the exact pair every
-// step, and the current is deposited from the pair itself.
+// in relative form holds, per axis, a reference offset o in [0, 1) -- along z
+// it moves with exactly the arithmetic of a drifting ion, across it stays
+// where the particle was placed, i.e. it is its ion's path -- plus the
+// departure dl from it, |dl| <= 1/2 (whole cells move between dl and the
+// reference cell, which is exact).  The position is c_ref + o + dl with c_ref =
+// c + r, c the stored cell (the one the electron is in, so that tiles and
+// stencils are as for any record) and r the shift this function returns; its
+// result is the electron's offset in cell c, in [0, 1), for the gather.  The
+// rounding of o + dl here does not accumulate: it is redone from the exact
+// pair every step, and the current is deposited from the pair itself.
 template <typename real>
 __host__ __device__ inline real rel_actual(real o, real dl, int &r)
 {
@@ -782,7 +782,18 @@ extern thread_local bool g_capture;
 // more of it on 2D grids of some thousand tiles: 256 x 2048 80 / 66 / 69, 256 x
 // 4096 118 / 105 / 108, 256 x 8192 200 / 186 / 188; with one stream 79 / 68 /
 // 65, 118 / 110 / 103, 198 / 187 / 183.)
-__device__ __forceinline__ void chain_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+//
+// A gradient's kernels on 2D grids of kEarlyNodes nodes or more do let the next
+// one in (Geom::early): most of their grids cover every SM evenly, and
+// gradients are run from programs with a stream per run, where launches take
+// longer.  128 x 1536 cells, a forward and a reverse run of 100 steps, early /
+// not: 14.1 / 14.7 ms on a process's sixth stream, 14.3 / 13.3 on its first.
+constexpr int64_t kEarlyNodes = 150000;  // (64 x 600 cells: 9.4 / 8.2 ms on any stream)
+__device__ __forceinline__ void chain_begin(int early)
+{
+    if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
 // (cluster: CTAs per thread-block cluster)
 template <typename... P, typename... A>
 inline void launch_clusters(unsigned cluster, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem,
@@ -860,7 +871,7 @@ struct ZeroArgs {
 // (returns the kernels it launches: none where a memset does it)
 template <typename real> int launch_zero(real *p, int64_t n, cudaStream_t s);
 // the same for two arrays in one launch (q: m bytes)
-template <typename real> void launch_zero2(real *p, int64_t n, unsigned char *q, int64_t m, cudaStream_t s);
+template <typename real> void launch_zero2(real *p, int64_t n, unsigned char *q, int64_t m, int early, cudaStream_t s);
 // SMs of the current device (cached per device)
 int device_sms();
 

@@ -13,7 +13,7 @@ template <typename real, int DIM, int S, int TX, int TY, int TZ, bool REL>
 __global__ void __launch_bounds__((BlockOf<real, DIM>::value), (MinBlocks<real, DIM>::value)) push_kernel(PushArgs<real> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    chain_begin();
+    chain_begin(a.g.early);
     for (int64_t t = blockIdx.x; t < a.g.ntiles; t += gridDim.x) push_tile<real, DIM, S, TX, TY, TZ, REL>(a, t, smem_raw);
 }
 
@@ -23,7 +23,7 @@ __global__ void __launch_bounds__((BlockOf<real, DIM>::value), (MinBlocks<real, 
     push_split_kernel(PushArgs<real> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    chain_begin();
+    chain_begin(a.g.early);
     push_tile<real, DIM, S, TX, TY, TZ, REL, kSplit>(a, (int64_t)(blockIdx.x / kSplit), smem_raw);
 }
 
@@ -33,7 +33,7 @@ template <typename real, int DIM, int S, int TX, int TY, int TZ, bool REL>
 __global__ void __launch_bounds__((BlockOf<real, DIM>::value)) ion_kernel(PushArgs<real> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    chain_begin();
+    chain_begin(a.g.early);
     for (int64_t t = blockIdx.x; t < a.g.ntiles; t += gridDim.x) ion_tile<real, DIM, S, TX, TY, TZ, REL>(a, t, smem_raw);
 }
 

@@ -1098,7 +1098,7 @@ __device__ __forceinline__ real rel_step(real dl, real d, int &fold)
 // the queue of leavers, before its current is deposited, so that the
 // momentum's registers are free by then.  Measured on a 128 x 128 x 256 slab
 // (33.6M electrons, gamma = 13): half of them still paired 1245 -> 955 us a
-// launch, all paired 703 -> 487 us (58% of the DRAM rate), from 1054M to 702M
+// launch, all paired 703 -> 487 us (57% of the DRAM rate), from 1054M to 702M
 // and 503M to 362M warp instructions.
 template <typename real, int DIM, int S, int TX, int TY, int TZ, bool REL, int SPLIT = 1>
 __device__ __forceinline__ void push_tile(const PushArgs<real> &a, const int64_t t, unsigned char *smem_raw)
